@@ -20,7 +20,8 @@
 //   gather  encode (warp = sample x 32 inputs, ballot into input words); drive
 //           and neuron update (warp = sample x 32 neurons over the sample's
 //           active words, each active row a 64-byte read), the sum in the
-//           order above: bit-exact with the oracle.
+//           order above: bit-exact with the oracle.  All steps run in one
+//           launch, a cluster per sample (k_rec_gather).
 //   dense   the drive of every (sample, neuron) as one tcgen05 GEMM per step,
 //           X[B][N] = S[B][K] * Wt[N][K]^T with S = (input spikes | previous
 //           hidden spikes) as bfloat16 0/1 and Wt = (W_ff ; W_rec) transposed,
@@ -82,9 +83,10 @@ struct RecConsts {
 struct RecBufs {
     uint16_t* S;             // [2][B][K]   spike operand of the dense form (bfloat16 0/1)
     int K;                   // n_in + n_hid rounded up to 64
-    const uint16_t* w_ff;    // [n_in][N] bfloat16
-    const uint16_t* w_rec;   // [N][N]
-    const uint16_t* w_out;   // [N][n_out]
+    int ldw;                 // row pitch of w_ff and w_rec: N rounded up to 8 (zeros past N)
+    const uint16_t* w_ff;    // [n_in][ldw] bfloat16; w_rec follows it in the same allocation
+    const uint16_t* w_rec;   // [N + 1][ldw], the last row zero
+    const uint16_t* w_out;   // [N + 1][n_out], the last row zero
     uint32_t* thr;           // [Bp/32][n_in][32] Poisson thresholds (sidx)
     uint64_t* seeds;         // [B]
     uint32_t* inb;           // [B][Iw]     input spikes of the step
@@ -198,7 +200,7 @@ __global__ void __launch_bounds__(256) k_rec_hidden(RecConsts c, RecBufs d, int 
         while (m) {
             const int a = w * 32 + __ffs(m) - 1;
             m &= m - 1;
-            x = __fadd_rn(x, bf16_value(d.w_ff[(size_t)a * c.N + jc]));
+            x = __fadd_rn(x, bf16_value(d.w_ff[(size_t)a * d.ldw + jc]));
         }
     }
     const uint32_t* hb = d.sh + ((size_t)prv * c.B + b) * c.Nw;
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(256) k_rec_hidden(RecConsts c, RecBufs d, int 
         while (m) {
             const int k = w * 32 + __ffs(m) - 1;
             m &= m - 1;
-            x = __fadd_rn(x, bf16_value(d.w_rec[(size_t)k * c.N + jc]));
+            x = __fadd_rn(x, bf16_value(d.w_rec[(size_t)k * d.ldw + jc]));
         }
     }
     const size_t q = sidx(b, jc, c.N);
@@ -227,6 +229,356 @@ __global__ void __launch_bounds__(256) k_rec_hidden(RecConsts c, RecBufs d, int 
     const uint32_t word = __ballot_sync(FULL, spk);
     if (lane == 0) d.sh[((size_t)cur * c.B + b) * c.Nw + jw] = word;
     if (vj) d.S[((size_t)prv * c.B + b) * d.K + c.n_in + j] = spk ? BF16_ONE : 0;   // next step's operand
+}
+
+// ---- gather form, all steps in one launch ----------------------------------
+// Samples do not interact, so a thread-block cluster of CS CTAs runs one
+// sample for all T steps: neuron state in registers, spikes and lists in shared
+// memory, no grid barrier and no launch per step.  CTA r owns neurons
+// [r*npc, (r+1)*npc).  Warps: nw neuron warps (VEC adjacent neurons per
+// thread), GSW that stream weight rows, one that adds the previous step's
+// readout (CTA 0), and the rest draw the CTA's share of the next step's inputs.
+// Per step:
+//   A  every warp takes the prefix sums over the spike words and lists its
+//      share of the active rows, ascending, inputs first (one stacked weight
+//      matrix, so a row index addresses either);
+//   B  the streaming warps copy the listed rows' column range into a ring of
+//      GR-row stages (16-byte asynchronous copies counted on an mbarrier; one
+//      bulk copy per row was as slow as no ring), and the neuron warps add them
+//      in order;
+//   C  neuron update; the spike words go to every CTA of the cluster.
+// What bounds it: the instructions of one warp in turn (about five per row and
+// neuron pair, the list, the draws; the SM's issue slots are a quarter busy)
+// and the rows' L2 round trip.  1024->512, B = 64, T = 100, a run with its
+// reads: 4.47 ms with the per-step kernels (45 us a step, one dependent load
+// per active row), 0.81 ms with sixteen rows in flight in each thread's
+// registers, 0.51 ms with the ring.  One neuron per thread, four, or more
+// drawing warps: 0.60, 0.55 and 0.51 ms.
+constexpr int GE = 8;                    // streaming, readout and drawing warps
+constexpr int GNW_MAX = 16;              // neuron warps
+constexpr int GSW = 4;                   // streaming warps, a stage each in turn
+constexpr int GR = 8;                    // rows per ring stage
+constexpr int GS_LOG = 4;                // ring stages at most, a power of two
+constexpr int GRING = 128 * 1024;        // ring bytes at most (at least two stages of the widest rows)
+constexpr int GCS_MAX = 8;               // CTAs per cluster (the portable size)
+
+struct GatherPlan {
+    int CS, VEC, npc, nw;                // CTAs per sample, neurons per thread and per CTA, neuron warps
+    int lgS, S;                          // ring stages (a power of two) and their logarithm
+    size_t o_bar, o_words, o_lst, o_thr, o_wo, smem;   // shared memory: ring, barriers, words, list,
+                                         // thresholds, W_out (o_wo = 0: read from global memory)
+};
+
+template <int VEC> struct RowVec;
+template <> struct RowVec<2> { using type = uint32_t; };
+template <> struct RowVec<4> { using type = uint2; };
+template <> struct RowVec<8> { using type = uint4; };
+
+// the row's VEC weights added to x
+template <int VEC>
+__device__ __forceinline__ void add_row(float (&x)[VEC], const typename RowVec<VEC>::type& r) {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(&r);
+#pragma unroll
+    for (int q = 0; q < VEC / 2; ++q) {
+        x[2 * q] = __fadd_rn(x[2 * q], __uint_as_float(w[q] << 16));
+        x[2 * q + 1] = __fadd_rn(x[2 * q + 1], __uint_as_float(w[q] & 0xFFFF0000u));
+    }
+}
+
+template <int VEC>
+__global__ void __launch_bounds__(32 * (GNW_MAX + GE), 1) k_rec_gather(RecConsts c, RecBufs d, GatherPlan g, int T,
+                                                                       uint32_t* err) {
+    extern __shared__ __align__(128) uint8_t gsm[];
+    const int IN = c.Iw + c.Nw;                            // words of a step: inputs, then hidden
+    uint64_t* const full = reinterpret_cast<uint64_t*>(gsm + g.o_bar);  // [S] rows landed; [S] stage free
+    uint64_t* const empty = full + g.S;
+    uint32_t* const words = reinterpret_cast<uint32_t*>(gsm + g.o_words);   // [2][IN]: input words of the step,
+                                                           // hidden words of the step before it
+    uint16_t* const lst = reinterpret_cast<uint16_t*>(gsm + g.o_lst);   // active rows, ascending
+    uint32_t* const thr = reinterpret_cast<uint32_t*>(gsm + g.o_thr);   // [n_in]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarp = blockDim.x >> 5;
+    const int b = blockIdx.x / g.CS, rank = blockIdx.x % g.CS;
+    const unsigned long long base = d.step[0];
+    const uint64_t seed = d.seeds[b];
+    const int j0 = rank * g.npc;                           // the CTA's first neuron
+    const int jl = tid * VEC, j = j0 + jl;                 // the thread's (neuron warps)
+    const bool is_neuron = warp < g.nw;
+    const bool live = is_neuron && jl < g.npc && j < c.N;
+    const int RB = g.npc * 2;                              // bytes of a ring row
+    const int cb = 2 * max(0, min(g.npc, d.ldw - j0));     // bytes of the CTA's columns (a multiple of 16)
+    const uint8_t* const wsrc = reinterpret_cast<const uint8_t*>(d.w_ff + (cb > 0 ? j0 : 0));
+    const size_t wpitch = (size_t)d.ldw * 2;
+    const uint32_t ring = su32(gsm);
+
+    float v[VEC], is[VEC];
+    uint32_t cnt[VEC];
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) {
+        const bool ok = live && j + q < c.N;
+        v[q] = ok ? d.v[sidx(b, j + q, c.N)] : 0.0f;
+        is[q] = ok ? d.i_syn[sidx(b, j + q, c.N)] : 0.0f;
+        cnt[q] = 0u;
+    }
+    for (int a = tid; a < c.n_in; a += blockDim.x) thr[a] = d.thr[sidx(b, a, c.n_in)];
+    for (int w = tid; w < c.Nw; w += blockDim.x)           // hidden spikes of the step before the first
+        words[c.Iw + w] = d.sh[((size_t)((base + 1ull) & 1ull) * c.B + b) * c.Nw + w];
+    float vout = 0.0f;                                     // CTA 0, readout warp: output `lane`
+    const bool streams = !is_neuron && warp < g.nw + GSW, reads_out = rank == 0 && warp == g.nw + GSW;
+    if (reads_out && lane < c.n_out) vout = d.v_out[(size_t)b * c.n_out + lane];
+    uint16_t* const wos = reinterpret_cast<uint16_t*>(gsm + g.o_wo);
+    if (g.o_wo && rank == 0)
+        for (int k = tid; k < (c.N + 1) * c.n_out; k += blockDim.x) wos[k] = d.w_out[k];
+    if (tid == 0) {
+        for (int s = 0; s < g.S; ++s) { mbar_init(&full[s], 32); mbar_init(&empty[s], (uint32_t)g.nw); }
+        snn::tc::mbar_fence_init();
+    }
+    if (g.CS == 1) __syncthreads();
+    else snn::tc::cluster_sync();                          // (every CTA runs before its memory is written)
+
+    // the input words of local step t
+    auto draw = [&](int t, int w0, int dw) {
+        uint32_t* out = words + (t & 1) * IN;
+        const unsigned long long tt = base + (unsigned long long)t;
+        for (int w = w0; w < c.Iw; w += dw) {
+            const int a = w * 32 + lane;
+            const bool s = a < c.n_in && snn::poisson_spike(seed, tt, c.n_in, a, thr[a]);
+            if (c.rec_input && a < c.n_in) d.raster_in[((size_t)t * c.B + b) * c.n_in + a] = s ? 1 : 0;
+            const uint32_t m = __ballot_sync(FULL, s);
+            if (g.CS == 1) {
+                if (lane == 0) out[w] = m;
+            } else if (lane < g.CS) {
+                snn::tc::st_cluster_u32(snn::tc::cluster_map(su32(out + w), (uint32_t)lane), m);
+            }
+        }
+    };
+    // v_out += sum over the hidden rows [h0, n) of the list of W_out, ascending
+    auto readout = [&](int h0, int n) {
+        for (int o0 = 0; o0 < c.n_out; o0 += 32) {
+            const int o = o0 + lane < c.n_out ? o0 + lane : c.n_out - 1;
+            float y = 0.0f;
+            const uint16_t* wo = (g.o_wo ? wos : d.w_out) + o;
+            for (int a = h0 & ~7; a < n; a += 32) {        // 32 loads in flight, added in order (entries outside
+                float wv[32];                              // [h0, n) read the zero row: the sum is never -0)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint4 i8 = *reinterpret_cast<const uint4*>(lst + a + 8 * e);
+                    const uint32_t ii[4] = {i8.x, i8.y, i8.z, i8.w};
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const int p = a + 8 * e + q - h0, row = (int)((ii[q >> 1] >> (16 * (q & 1))) & 0xFFFFu);
+                        const int k = (unsigned)p < (unsigned)(n - h0) ? row - c.n_in : c.N;   // (a load each, no branch)
+                        wv[8 * e + q] = bf16_value(wo[k * c.n_out]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 32; ++q) y = __fadd_rn(y, wv[q]);
+            }
+            if (o0 == 0) {
+                vout = __fadd_rn(vout, y);
+            } else if (o0 + lane < c.n_out) {
+                float* p = d.v_out + (size_t)b * c.n_out + o;
+                *p = __fadd_rn(*p, y);
+            }
+        }
+    };
+
+    draw(0, rank + g.CS * warp, g.CS * nwarp);
+    if (g.CS == 1) __syncthreads();
+    else snn::tc::cluster_sync();
+    int it = 0;                                            // ring stages used so far (the same in every warp)
+    bool ok = true;                                        // no wait has given up
+    int h0;                                                // list position of the first hidden row
+    for (int t = 0; t <= T; ++t) {                         // t = T: the last step's readout only
+        // ---- A: the list
+        const uint32_t* wt = words + (t & 1) * IN;
+        // each lane counts two words of a 64-word chunk, both scanned in one word
+        // (a chunk half holds at most 1024 rows)
+        int n = 0;
+        for (int q0 = 0; q0 < IN; q0 += 64) {
+            const uint32_t wa = q0 + lane < IN ? wt[q0 + lane] : 0u;
+            const uint32_t wb = q0 + 32 + lane < IN ? wt[q0 + 32 + lane] : 0u;
+            const int k = __popc(wa) | (__popc(wb) << 16);
+            int x = k;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(FULL, x, o);
+                if (lane >= o) x += y;
+            }
+            const int tot = __shfl_sync(FULL, x, 31), na = n + (tot & 0xFFFF);
+            x -= k;
+            const int sa = n + (x & 0xFFFF), sb = na + (x >> 16);   // rows before each lane's two words
+            const int hw = c.Iw - q0;
+            if (hw >= 0 && hw < 64) h0 = __shfl_sync(FULL, hw < 32 ? sa : sb, hw & 31);
+            for (int w = warp; w < 64 && q0 + w < IN; w += nwarp) {   // this warp's words
+                const uint32_t m = __shfl_sync(FULL, w < 32 ? wa : wb, w & 31);
+                const int st = __shfl_sync(FULL, w < 32 ? sa : sb, w & 31);
+                const int g32 = (q0 + w) * 32 + lane;
+                if ((m >> lane) & 1u)
+                    lst[st + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(q0 + w < c.Iw ? g32 : g32 - 32 * c.Iw + c.n_in);
+            }
+            n = na + (tot >> 16);
+        }
+        const int nst = (n + GR - 1) / GR;                 // ring stages; the last padded with the zero row
+        if (warp == 0 && n + lane < nst * GR) lst[n + lane] = (uint16_t)(c.n_in + c.N);
+        __syncthreads();
+        if (t > 0 && reads_out) readout(h0, n);            // of the previous step
+        if (t == T) break;
+        if (streams) {
+            // ---- B: the listed rows into the ring
+            // stage i belongs to warp i mod ns: S is a multiple of ns, so a slot is
+            // refilled by one warp, which sees every phase of its barrier in turn
+            const int ns = min(GSW, g.S), ws = warp - g.nw;
+            for (int k = ws < ns ? (ws - it) & (ns - 1) : nst; k < nst && cb > 0; k += ns) {
+                const int i = it + k, s = i & (g.S - 1);
+                uint32_t ii[GR / 2];
+#pragma unroll
+                for (int q = 0; q < GR / 8; ++q)
+                    *reinterpret_cast<uint4*>(ii + 4 * q) = *reinterpret_cast<const uint4*>(lst + k * GR + 8 * q);
+                const uint8_t* src[GR];                    // all addresses first: the copies then issue back to back
+#pragma unroll
+                for (int q = 0; q < GR; ++q)
+                    src[q] = wsrc + (size_t)((ii[q >> 1] >> (16 * (q & 1))) & 0xFFFFu) * wpitch;
+                if (i >= g.S && ok) ok = mbar_wait(&empty[s], ((i >> g.lgS) - 1) & 1);
+                ok = __all_sync(FULL, ok ? 1 : 0) != 0;
+                if (!ok) break;
+                for (int x = 16 * lane; x < cb; x += 512)
+#pragma unroll
+                    for (int q = 0; q < GR; ++q) snn::tc::cp_async16(ring + (uint32_t)((s * GR + q) * RB + x), src[q] + x);
+                snn::tc::cp_async_arrive(&full[s]);
+            }
+        } else if (!is_neuron) {
+            if (t + 1 < T && !reads_out)
+                draw(t + 1, rank + g.CS * (warp - g.nw - GSW - (rank == 0 ? 1 : 0)), g.CS * (GE - GSW - (rank == 0 ? 1 : 0)));
+        } else {
+            using V = typename RowVec<VEC>::type;
+            float x[VEC];
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) x[q] = 0.0f;
+            for (int k = 0; k < nst && cb > 0; ++k) {
+                const int i = it + k, s = i & (g.S - 1);
+                if (ok) ok = mbar_wait(&full[s], (i >> g.lgS) & 1);
+                const uint8_t* src = gsm + s * GR * RB + tid * (VEC * 2);
+                constexpr int U = VEC == 8 ? 4 : GR;       // rows loaded together (registers)
+#pragma unroll
+                for (int u = 0; u < GR; u += U) {
+                    V r[U];
+#pragma unroll
+                    for (int q = 0; q < U; ++q) r[q] = *reinterpret_cast<const V*>(src + (u + q) * RB);
+                    if (u + U == GR) {
+                        __syncwarp();
+                        if (lane == 0) snn::tc::mbar_arrive(&empty[s]);
+                    }
+#pragma unroll
+                    for (int q = 0; q < U; ++q) add_row<VEC>(x, r[q]);
+                }
+            }
+            // ---- C: synapse and neuron, spike words to the whole cluster
+            uint32_t bits = 0u;
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) {
+                is[q] = __fadd_rn(__fmul_rn(c.a_syn, is[q]), x[q]);
+                v[q] = __fadd_rn(__fmul_rn(c.a_mem, v[q]), is[q]);
+                const bool spk = live && j + q < c.N && v[q] >= c.v_thresh;
+                if (spk) { v[q] = c.v_reset; ++cnt[q]; bits |= 1u << q; }
+                if (c.rec_raster && live && j + q < c.N)
+                    d.raster_h[((size_t)t * c.B + b) * c.N + j + q] = spk ? 1 : 0;
+            }
+            uint32_t word = bits << (jl & 31);
+#pragma unroll
+            for (int o = 1; o < 32 / VEC; o <<= 1) word |= __shfl_xor_sync(FULL, word, o);
+            uint32_t* const wnext = words + ((t + 1) & 1) * IN + c.Iw;
+            const int w = j >> 5;
+            if ((jl & 31) == 0 && jl < g.npc && w < c.Nw) {
+                if (g.CS == 1) {
+                    wnext[w] = word;
+                } else {
+                    for (int k = 0; k < g.CS; ++k)
+                        snn::tc::st_cluster_u32(snn::tc::cluster_map(su32(wnext + w), (uint32_t)k), word);
+                }
+            }
+        }
+        if (cb > 0) it += nst;
+        if (g.CS == 1) __syncthreads();
+        else snn::tc::cluster_sync();
+    }
+    if (!ok && lane == 0) atomicOr(err, 1u);
+    if (streams) snn::tc::cp_async_wait_all();             // no copy lands after the CTA has left
+
+    // ---- the state back; the last step's spikes as words and as the operand of
+    // the step that follows
+    const unsigned long long last = base + (unsigned long long)T - 1ull;
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) {
+        if (!live || j + q >= c.N) continue;
+        d.v[sidx(b, j + q, c.N)] = v[q];
+        d.i_syn[sidx(b, j + q, c.N)] = is[q];
+        d.counts[sidx(b, j + q, c.N)] = cnt[q];
+        const uint32_t m = words[(T & 1) * IN + c.Iw + ((j + q) >> 5)];
+        d.S[((size_t)((last + 1ull) & 1ull) * c.B + b) * d.K + c.n_in + j + q] = (m >> ((j + q) & 31)) & 1u ? BF16_ONE : 0;
+    }
+    if (rank == 0)
+        for (int w = tid; w < c.Nw; w += blockDim.x)
+            d.sh[((size_t)(last & 1ull) * c.B + b) * c.Nw + w] = words[(T & 1) * IN + c.Iw + w];
+    if (reads_out && lane < c.n_out) d.v_out[(size_t)b * c.n_out + lane] = vout;
+}
+
+// The gather form's plan, or CS = 0 where its limits do not hold (the per-step
+// kernels then run).  Clusters as wide as the SMs allow while a CTA keeps at
+// least 256 neurons: a wider cluster shares the row loads among more SMs but
+// not their latency.  Then the narrowest vector that GNW_MAX warps cover.
+GatherPlan gather_plan(const RecConsts& c, int sms) {
+    GatherPlan g{};
+    if ((long long)c.n_in + c.N > 65535) return g;         // 16-bit row indices (the zero row's included)
+    int cs = 1;
+    while (cs < GCS_MAX && (((c.N + cs - 1) / cs > 32 * GNW_MAX * 8) ||
+                            ((long long)c.B * cs * 2 <= sms && (c.N + 2 * cs - 1) / (2 * cs) >= 256)))
+        cs *= 2;
+    const int npc = ((c.N + cs - 1) / cs + 31) / 32 * 32;
+    int vec = 2;
+    while (vec < 8 && npc > 32 * GNW_MAX * vec) vec *= 2;
+    if (npc > 32 * GNW_MAX * vec) return g;
+    const int stage = GR * npc * 2;
+    g.lgS = GS_LOG;                                        // npc <= 4096: at least two stages
+    while ((stage << g.lgS) > GRING) --g.lgS;
+    g.S = 1 << g.lgS;
+    auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
+    g.o_bar = (size_t)g.S * stage;
+    g.o_words = g.o_bar + (size_t)2 * g.S * 8;
+    g.o_lst = up(g.o_words + (size_t)2 * (c.Iw + c.Nw) * 4);
+    g.o_thr = up(g.o_lst + (size_t)(c.n_in + c.N + 40) * 2);
+    g.smem = g.o_thr + (size_t)c.n_in * 4;
+    if (g.smem > 224 * 1024) return g;
+    // the cluster barrier's acquire drops L1, so W_out is kept in shared memory where it fits
+    const size_t wo = up((size_t)(c.N + 1) * c.n_out * 2);
+    if (up(g.smem) + wo <= 224 * 1024) {
+        g.o_wo = up(g.smem);
+        g.smem = g.o_wo + wo;
+    }
+    g.VEC = vec;
+    g.npc = npc;
+    g.nw = (npc + 32 * vec - 1) / (32 * vec);
+    g.CS = cs;
+    return g;
+}
+
+cudaError_t launch_gather(const RecConsts& c, const RecBufs& d, const GatherPlan& g, int T, uint32_t* err,
+                          cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(c.B * g.CS));
+    cfg.blockDim = dim3((unsigned)(32 * (g.nw + GE)));
+    cfg.dynamicSmemBytes = g.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)g.CS;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    auto kern = g.VEC == 2 ? k_rec_gather<2> : g.VEC == 4 ? k_rec_gather<4> : k_rec_gather<8>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchKernelEx(&cfg, kern, c, d, g, T, err);
 }
 
 // 32 consecutive columns col0.. (nu of them live) of the spike operand of slot
@@ -663,14 +1015,14 @@ __global__ void k_rec_put_spikes(RecConsts c, RecBufs d, const uint8_t* __restri
 // on the hidden columns; 0 elsewhere
 __global__ void k_rec_pack(const uint16_t* __restrict__ w_ff, const uint16_t* __restrict__ w_rec,
                            const uint16_t* __restrict__ w_out, uint16_t* __restrict__ wt, int n_in, int N,
-                           int n_out, int K, int R0, int rows) {
+                           int ldw, int n_out, int K, int R0, int rows) {
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (size_t)rows * K) return;
     const int j = (int)(idx / K), k = (int)(idx % K);
     uint16_t w = 0;
     if (j < N) {
-        if (k < n_in) w = w_ff[(size_t)k * N + j];
-        else if (k < n_in + N) w = w_rec[(size_t)(k - n_in) * N + j];
+        if (k < n_in) w = w_ff[(size_t)k * ldw + j];
+        else if (k < n_in + N) w = w_rec[(size_t)(k - n_in) * ldw + j];
     } else if (j >= R0 && j < R0 + n_out && k >= n_in && k < n_in + N) {
         w = w_out[(size_t)(k - n_in) * n_out + (j - R0)];
     }
@@ -691,7 +1043,7 @@ bool finite_pos(float x) { return std::isfinite(x) && x > 0.0f; }
 struct snn_rec {
     snn_rec_spec spec{};
     int device = 0;
-    uint16_t* w_ff = nullptr;
+    uint16_t* w_ff = nullptr;          // W_ff, then W_rec (w_rec points into it)
     uint16_t* w_rec = nullptr;
     uint16_t* w_out = nullptr;
     uint16_t* wt = nullptr;            // [wt_rows][K] stacked transposed weights of the dense form
@@ -758,6 +1110,7 @@ void free_batch(snn_rec* r) {
     r->d = RecBufs{};
     r->d.w_ff = keep.w_ff; r->d.w_rec = keep.w_rec; r->d.w_out = keep.w_out; r->d.step = keep.step;
     r->d.K = keep.K;
+    r->d.ldw = keep.ldw;
     r->rates_stage = nullptr; r->seeds_stage = nullptr;
     r->raster_h_cap = r->raster_in_cap = 0;
     r->B = 0;
@@ -841,11 +1194,16 @@ snn_status snn_rec_create(const snn_rec_spec* spec, snn_rec** out) {
     r->spec = s;
     r->spec.w_ff = r->spec.w_rec = r->spec.w_out = nullptr;   // copies are owned below
     cudaError_t e = cudaGetDevice(&r->device);
-    const size_t nff = (size_t)s.n_in * s.n_hid, nrec = (size_t)s.n_hid * s.n_hid,
-                 nout = (size_t)s.n_hid * s.n_out;
-    if (e == cudaSuccess) e = dalloc(&r->w_ff, nff);
-    if (e == cudaSuccess) e = dalloc(&r->w_rec, nrec);
-    if (e == cudaSuccess) e = dalloc(&r->w_out, nout);
+    const size_t nout = (size_t)s.n_hid * s.n_out;
+    // W_ff and W_rec stacked in one allocation, rows padded to whole 16-byte
+    // vectors, with a row of zeros after them (and after W_out): the gather form
+    // indexes them as one matrix and pads its lists with the zero row
+    const size_t ldw = ((size_t)s.n_hid + 7) / 8 * 8, nw = ((size_t)s.n_in + s.n_hid + 1) * ldw;
+    const size_t row = (size_t)s.n_hid * 2;
+    r->d.ldw = (int)ldw;
+    if (e == cudaSuccess) e = dalloc(&r->w_ff, nw);
+    if (e == cudaSuccess) r->w_rec = r->w_ff + (size_t)s.n_in * ldw;
+    if (e == cudaSuccess) e = dalloc(&r->w_out, nout + s.n_out);
     r->K = (s.n_in + s.n_hid + GBK - 1) / GBK * GBK;
     if (e == cudaSuccess) e = dalloc(&r->step, 2);
     r->geom.ntn_drive = (s.n_hid + GBN - 1) / GBN;
@@ -860,14 +1218,22 @@ snn_status snn_rec_create(const snn_rec_spec* spec, snn_rec** out) {
     if (e == cudaSuccess) e = dalloc(&r->act_dev, 1);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&r->act_host, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r->act_ev, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMemcpy(r->w_ff, s.w_ff, nff * 2, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(r->w_rec, s.w_rec, nrec * 2, cudaMemcpyHostToDevice);
+    if (ldw == (size_t)s.n_hid) {
+        if (e == cudaSuccess) e = cudaMemset(r->w_ff + (nw - ldw), 0, ldw * 2);
+        if (e == cudaSuccess) e = cudaMemcpy(r->w_ff, s.w_ff, s.n_in * row, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(r->w_rec, s.w_rec, s.n_hid * row, cudaMemcpyHostToDevice);
+    } else {
+        if (e == cudaSuccess) e = cudaMemset(r->w_ff, 0, nw * 2);
+        if (e == cudaSuccess) e = cudaMemcpy2D(r->w_ff, ldw * 2, s.w_ff, row, row, s.n_in, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy2D(r->w_rec, ldw * 2, s.w_rec, row, row, s.n_hid, cudaMemcpyHostToDevice);
+    }
+    if (e == cudaSuccess) e = cudaMemset(r->w_out + nout, 0, (size_t)s.n_out * 2);
     if (e == cudaSuccess) e = cudaMemcpy(r->w_out, s.w_out, nout * 2, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(r->step, 0, 16);
     if (e == cudaSuccess) {
         const size_t n = (size_t)r->wt_rows * r->K;
         k_rec_pack<<<(unsigned)((n + 255) / 256), 256>>>(r->w_ff, r->w_rec, r->w_out, r->wt, s.n_in, s.n_hid,
-                                                         s.n_out, r->K, r->geom.ntn_drive * GBN, r->wt_rows);
+                                                         r->d.ldw, s.n_out, r->K, r->geom.ntn_drive * GBN, r->wt_rows);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -894,7 +1260,6 @@ snn_status snn_rec_destroy(snn_rec* r) {
     if (r->last) cudaStreamSynchronize(r->last);
     free_batch(r);
     if (r->w_ff) cudaFree(r->w_ff);
-    if (r->w_rec) cudaFree(r->w_rec);
     if (r->w_out) cudaFree(r->w_out);
     if (r->step) cudaFree(r->step);
     if (r->wt) cudaFree(r->wt);
@@ -998,7 +1363,11 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
     // the tensor form draws each next step's inputs in the product's epilogue,
     // unless the input raster is recorded
     const bool fuse_enc = dense && !c.rec_input;
-    for (int t = 0; t < T; ++t) {
+    // the gather form: all steps in one launch where its limits hold (a profiled
+    // run keeps the per-step launches that its report counts)
+    const GatherPlan plan = dense || profile || T == 0 ? GatherPlan{} : gather_plan(c, r->num_sms);
+    if (plan.CS) REC_TRY(r, launch_gather(c, d, plan, T, r->dev_err, st));
+    for (int t = 0; t < (plan.CS ? 0 : T); ++t) {
         if (!fuse_enc || t == 0) {
             mark(SNN_REC_KERNEL_ENCODE, true);
             k_rec_encode<<<(unsigned)((enc_warps + 7) / 8), 256, 0, st>>>(c, d, t, dense);

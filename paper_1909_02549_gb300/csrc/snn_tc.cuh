@@ -47,7 +47,8 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
 // Waits for the phase with the given parity to complete; false once limit_ns
 // of %globaltimer have passed (the caller then reports an error and leaves).
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, unsigned long long limit_ns) {
-    if (mbar_try(b, parity)) return true;
+    for (int i = 0; i < 64; ++i)                          // (reading the timer costs far more than a try)
+        if (mbar_try(b, parity)) return true;
     const unsigned long long t0 = now_ns();
     for (;;) {
         for (int i = 0; i < 64; ++i)
@@ -63,6 +64,16 @@ __device__ __forceinline__ void tma_2d(void* dst, const CUtensorMap* tm, int c0,
                  "[%0], [%1, {%2, %3}], [%4];"
                  :: "r"(su32(dst)), "l"((uint64_t)tm), "r"(c0), "r"(c1), "r"(su32(bar)) : "memory");
 }
+// 16-byte asynchronous copies (through L2 only); cp_async_arrive makes the
+// mbarrier's current phase wait for the calling thread's copies so far (one
+// arrival of its expected count).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(src));
+}
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" :: "r"(su32(bar)) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // Shared-memory matrix descriptor of a K-major tile with 128-byte rows and the
 // 128-byte swizzle: groups of 8 rows 1024 bytes apart (SBO), version 1,
 // swizzle mode 2.  Advancing K by 16 elements adds 32 bytes (2 in the address
@@ -125,6 +136,9 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t saddr, uint32_t rank) {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
     return r;
+}
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
 }
 __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
     float4 v;
