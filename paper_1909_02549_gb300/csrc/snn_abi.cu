@@ -178,7 +178,7 @@ snn_status alloc_batch(snn_net* n, int B) {
     CUDA_TRY(n, dalloc(&d.x_pre, snn::XPRE_SLOTS * (size_t)B * NI));
     CUDA_TRY(n, dalloc(&d.inb, 2 * (size_t)B * Iw));
     CUDA_TRY(n, dalloc(&d.preT, snn::PRET_SLOTS * NI * Bw));
-    CUDA_TRY(n, dalloc(&d.act_idx, 2 * (size_t)B * NI));
+    CUDA_TRY(n, dalloc(&d.act_idx, 2 * (size_t)B * ((NI + 7) & ~(size_t)7)));
     CUDA_TRY(n, dalloc(&d.act_cnt, 2 * (size_t)B));
     CUDA_TRY(n, dalloc(&d.v_e, (size_t)B * N));
     CUDA_TRY(n, dalloc(&d.v_i, (size_t)B * N));
@@ -260,6 +260,19 @@ snn::Consts make_consts(const snn_net* n, int B, float dt, int learn, int reduce
     c.neuron = s.neuron;
     c.wmaster = s.wmaster;
     return c;
+}
+
+// One step of the per-step and graph forms: a launch over column tiles, or the
+// separate encode, neuron and update kernels where that does not apply (the
+// post-triggered rule, layers whose tile does not fit shared memory) and in
+// profiled runs, whose report counts them.
+cudaError_t step_launches(const snn::Consts& c, const snn::Bufs& d, int t, int T, cudaStream_t s, snn::Prof* pp) {
+    int used = 0;
+    if (!pp) {
+        const cudaError_t e = snn::launch_cols_step(c, d, t, T, s, &used);
+        if (e != cudaSuccess || used) return e;
+    }
+    return snn::launch_step(c, d, t, s, pp);
 }
 
 snn::Bufs run_bufs(const snn_net* n) { return n->d; }
@@ -610,7 +623,7 @@ snn_status snn_run(snn_net* n, const float* rates, const uint64_t* seeds, int B,
     }
     if (mode == SNN_MODE_TENSOR) CUDA_TRY(n, snn::launch_tensor_begin(c, d, n->tb, st, pp));
     if (mode == SNN_MODE_STEP) {
-        for (int t = 0; t < T; ++t) CUDA_TRY(n, snn::launch_step(c, d, t, st, pp));
+        for (int t = 0; t < T; ++t) CUDA_TRY(n, step_launches(c, d, t, T, st, pp));
     } else if (mode == SNN_MODE_GRAPH || mode == SNN_MODE_TENSOR) {
         const bool tensor = mode == SNN_MODE_TENSOR;
         GraphKey key;
@@ -631,7 +644,7 @@ snn_status snn_run(snn_net* n, const float* rates, const uint64_t* seeds, int B,
             if (pp) pp->capturing = true;
             for (int t = 0; t < T && le == cudaSuccess; ++t)
                 le = tensor ? snn::launch_tensor_step(c, d, n->tb, t, n->cap, pp)
-                            : snn::launch_step(c, d, t, n->cap, pp);
+                            : step_launches(c, d, t, T, n->cap, pp);
             if (pp) pp->capturing = false;
             cudaError_t ee = cudaStreamEndCapture(n->cap, &g);
             CUDA_TRY(n, le);

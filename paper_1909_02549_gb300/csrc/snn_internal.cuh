@@ -137,7 +137,7 @@ struct Bufs {
     float* x_pre;        // [XPRE_SLOTS][B][n_in] presynaptic traces after step tt (slot tt % 3)
     uint32_t* inb;       // [2][B][Iw]   input spikes of step tt, sample-major bits
     uint32_t* preT;      // [PRET_SLOTS][n_in][Bw] input spikes of step tt, input-major bits (slot tt % 4)
-    uint16_t* act_idx;   // [2][B][n_in] active inputs of step tt, ascending (persistent form)
+    uint16_t* act_idx;   // [2][B][n_in] active inputs of step tt, ascending (the column-tile step pads rows to 8)
     uint32_t* act_cnt;   // [2][B]
     float* v_e;          // [B][N]
     float* v_i;          // [B][N]
@@ -265,6 +265,9 @@ cudaError_t launch_begin_run(const Consts& c, const Bufs& d, const float* rates,
                              const uint64_t* seeds, int episodic, int T, cudaStream_t s,
                              Prof* prof);
 cudaError_t launch_step(const Consts& c, const Bufs& d, int t_local, cudaStream_t s, Prof* prof);
+// The same step as one launch over column tiles (snn_cols.cu), t_local of a run
+// of T steps in order; *used = 0 (and nothing launched) where it does not apply.
+cudaError_t launch_cols_step(const Consts& c, const Bufs& d, int t_local, int T, cudaStream_t s, int* used);
 cudaError_t launch_extract(const Consts& c, const Bufs& d, int field, void* scratch,
                            cudaStream_t s);
 

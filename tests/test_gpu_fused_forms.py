@@ -1,0 +1,61 @@
+"""The fused forms (a sample in one CTA or cluster for a whole run; a step in one
+launch over column tiles) at the sizes where their splits change: bit for bit
+against the oracle."""
+import numpy as np
+import pytest
+
+from test_gpu_rec import _built, assert_same, dev, oracle_run, snn, workload  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("B,NI,N,NO,T", [
+    (1, 40, 1100, 10, 40),     # clusters of four CTAs, the last with a short column range
+    (2, 1030, 64, 40, 40),     # more outputs than lanes, two warps of neurons, ragged input words
+    (153, 33, 520, 3, 20),     # one CTA per sample, more samples than SMs
+    (2, 64, 4200, 10, 12),     # clusters of eight
+    (80, 24, 4200, 10, 6),     # two CTAs by the layer's width, eight neurons per thread
+])
+def test_rec_gather_one_launch(B, NI, N, NO, T):
+    """Two runs, the second continuing, and the tensor form's operands left so
+    that a per-step (profiled) run continues too."""
+    p, r, s, wf, wr, wo = workload(B, NI, N, NO, seed=B)
+    net = snn().RecNetwork(p, wf, wr, wo)
+    st, rh, ri = oracle_run(p, r, s, wf, wr, wo, T)
+    assert rh.sum() > 0
+    net.run(dev(r), dev(s), T, record=True, record_input=True, form="gather")
+    assert_same(net, st, rh, ri)
+    for profile in (False, True):
+        st, rh, ri = oracle_run(p, r, s, wf, wr, wo, 3, st=st, episodic=False)
+        net.run(dev(r), dev(s), 3, continue_=True, record=True, record_input=True, form="gather", profile=profile)
+        assert_same(net, st, rh, ri)
+    net.close()
+
+
+@pytest.mark.parametrize("B,NI,N,T,reduce", [
+    (3, 7, 1, 60, "mean"),         # one column, fewer inputs than a list's load
+    (37, 100, 6007, 8, "sum"),     # 16 columns a block, rows that are not 16-byte aligned, a short last tile
+    (65, 30, 2504, 12, "max"),     # eight columns a block, three mask words
+    (257, 9, 130, 25, "mean"),     # four columns a block, nine mask words, a last tile of two
+])
+def test_column_tile_step(B, NI, N, T, reduce):
+    """The column-tile step at the edges of its tiles, learning and frozen, and
+    handing over to the persistent form and to the separate (profiled) kernels
+    in continuing runs."""
+    import test_gpu_parity as tp
+    p, r, s, w = tp.synth.fig1_workload(B, N, n_in=NI)
+    p.update(theta_plus=0.05, w_ei=22.5, w_ie=-0.5, e_thresh=-64.0)     # some inhibition and adaptation
+    tp.parity_all_modes(p, r, s, w, T, learn=False, modes=("graph",))
+    st, rec = tp.oracle_run(p, r, s, w, T, reduce=reduce)
+    assert rec.raster_e.sum() > 0 and np.abs(st.w - w).max() > 0
+    net, g = tp.gpu_run(p, r, s, w, T, reduce=reduce, mode="graph")
+    tp.assert_parity(g, st, rec)
+    for mode in ("step", "persistent", "graph"):
+        st, rec = tp.oracle_run(p, r, s, w, 3, reduce=reduce, st=st, episodic=False)
+        net, g = tp.gpu_run(p, r, s, w, 3, reduce=reduce, mode=mode, net=net, continue_=True)
+        tp.assert_parity(g, st, rec)
+    st, rec = tp.oracle_run(p, r, s, w, 2, reduce=reduce, st=st, episodic=False)
+    net.run(dev(r), dev(s), 2, reduce=reduce, mode="graph", continue_=True, profile=True)
+    assert np.array_equal(net.weights(), st.w) and np.array_equal(net.read("v_exc"), st.v_e)
+    net.close()
