@@ -32,6 +32,10 @@
 #include "snn_internal.cuh"
 
 namespace snn {
+
+// The learning-off form (snn_infer.cu); *used = 0 where it does not apply.
+cudaError_t launch_infer(const Consts& c, const Bufs& d, int T, cudaStream_t s, int* used);
+
 namespace {
 
 constexpr int PT = 1024;                   // threads per CTA (fewer, with more registers each, ran slower)
@@ -1917,6 +1921,14 @@ cudaError_t launch_persistent(const Consts& c, const Bufs& d, int T, cudaStream_
         attr = L.bytes;
     }
     lock.unlock();
+    if (!c.learn) {   // nothing couples the samples: a CTA per sample
+        e = prof_start(prof, SNN_KERNEL_PERSISTENT, s);
+        if (e != cudaSuccess) return e;
+        e = launch_infer(c, d, T, s, used);
+        if (e != cudaSuccess) return e;
+        if (*used) return prof_stop(prof, s);
+        if (prof) prof->n -= 1;               // not taken: the event is recorded again below
+    }
     Consts cc = c;
     Bufs dd = d;
     int TT = T;

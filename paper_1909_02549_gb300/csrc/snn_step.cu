@@ -429,6 +429,11 @@ cudaError_t launch_begin_run(const Consts& c, const Bufs& d, const float* rates,
     return prof_stop(prof, s);
 }
 
+cudaError_t launch_colscale(const Consts& c, const Bufs& d, cudaStream_t s) {
+    k_colscale<<<(c.N + 255) / 256, 256, 0, s>>>(c, d);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_step(const Consts& c, const Bufs& d, int t_local, cudaStream_t s, Prof* prof) {
     PROF_TRY(prof_start(prof, SNN_KERNEL_ENCODE, s));
     const size_t warps = (size_t)c.B * c.Iw;
@@ -436,10 +441,7 @@ cudaError_t launch_step(const Consts& c, const Bufs& d, int t_local, cudaStream_
     PROF_TRY(cudaGetLastError());
     PROF_TRY(prof_stop(prof, s));
     const size_t bn = (size_t)c.B * c.N;
-    if (c.wprec == SNN_W_FP8E4M3) {
-        k_colscale<<<(c.N + 255) / 256, 256, 0, s>>>(c, d);
-        PROF_TRY(cudaGetLastError());
-    }
+    if (c.wprec == SNN_W_FP8E4M3) PROF_TRY(launch_colscale(c, d, s));
     PROF_TRY(prof_start(prof, SNN_KERNEL_NEURON, s));
     k_neuron<<<(unsigned)((bn + 255) / 256), 256, 0, s>>>(c, d, t_local);
     PROF_TRY(cudaGetLastError());

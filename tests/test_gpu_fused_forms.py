@@ -59,3 +59,31 @@ def test_column_tile_step(B, NI, N, T, reduce):
     net.run(dev(r), dev(s), 2, reduce=reduce, mode="graph", continue_=True, profile=True)
     assert np.array_equal(net.weights(), st.w) and np.array_equal(net.read("v_exc"), st.v_e)
     net.close()
+
+
+@pytest.mark.parametrize("B,NI,N,T", [
+    (3, 70, 31, 40),         # fewer neurons than a warp, warps without neurons
+    (200, 1100, 512, 25),    # the widest layer at one neuron per thread, 35 input words
+    (5, 784, 2049, 40),      # four neurons per thread, one of them past a boundary
+    (2, 784, 8192, 20),      # the widest layer at eight
+])
+@pytest.mark.parametrize("wprec", [0, 1, 2])
+def test_learning_off_sample_per_cta(B, NI, N, T, wprec):
+    """The persistent mode with learning off, after a learning run has left
+    traces, so that inputs that never spike decay too; a second continuing run
+    has other rates, some of them all zero."""
+    import test_gpu_parity as tp
+    p, r, s, w = tp.synth.workload(B, N, NI)
+    net, g = tp.gpu_run(p, r, s, w, 5, mode="graph", wprec=wprec)
+    st, rec = tp.oracle_run(p, r, s, w, 5, wprec=wprec)
+    tp.assert_parity(g, st, rec)
+    r2 = np.roll(r, 7, axis=1) * np.float32(2)
+    r2[0] = 0
+    for rates, steps in ((r, T), (r2, 13)):
+        st, rec = tp.oracle_run(p, rates, s, w, steps, learn=False, st=st, episodic=False, wprec=wprec)
+        net, g = tp.gpu_run(p, rates, s, w, steps, learn=False, mode="persistent", net=net, continue_=True)
+        tp.assert_parity(g, st, rec)
+    st, rec = tp.oracle_run(p, r, s, w, 4, st=st, episodic=False, wprec=wprec)
+    net, g = tp.gpu_run(p, r, s, w, 4, mode="graph", net=net, continue_=True)
+    tp.assert_parity(g, st, rec)
+    net.close()
