@@ -1,7 +1,7 @@
 // Frozen presentations, one sample per CTA: with learning off the samples of a
 // batch do not interact, so a CTA runs its sample for many steps with the
 // neurons' state in registers and no exchange with other CTAs.  Used by the
-// learning-off runs of the persistent mode.
+// learning-off runs of the persistent mode and by the serving loop.
 //
 // Inputs whose rate is zero never spike and are left out once, at the start:
 // the draws and lists below run over the live inputs, ascending.  Per step:

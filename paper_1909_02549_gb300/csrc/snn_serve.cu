@@ -16,24 +16,31 @@
 // counts equal those of running it alone.
 //
 // The work of a call scales with the live slots, not with the capacity: one
-// launch of k_serve_chunk runs up to k steps with one CTA per live slot (its
-// list is uploaded with the call), and the all-but-self inhibition of a slot
-// is a count inside its CTA.  Calls do not wait for the device: the host knows
-// each slot's remaining steps, so it retires and backfills without reading
-// anything back; the finished requests' counts are gathered into a ring of
-// result rows and copied to pinned memory behind an event, and
-// snn_serve_poll hands out those whose copy has landed.  Per-call host staging
-// (admitted rates, slot lists) rotates through a few pinned buffers, each
-// reused only after the call that last used it has finished on the device,
-// which also bounds how far the host runs ahead.
+// launch of k_serve_chunk runs up to k steps with one CTA per live slot, and
+// the all-but-self inhibition of a slot is a count inside its CTA.  Calls do not
+// wait for the device: the host knows each slot's remaining steps, so it retires
+// and backfills without reading anything back, and snn_serve_poll hands out the
+// requests whose call has finished (an event).
+//
+// A call is one launch (two when it admits): the kernels read the call's
+// admissions and slot list in pinned host memory, and a slot that ends in the
+// call writes its counts to a pinned result row itself.  With 512 requests of 50
+// to 500 steps, 400 neurons, k = 10, a call took 56 us of host time (copies of
+// its lists, a gather launch, a copy per finished row, scans over all slots) and
+// its kernel 43 us; now 29 us on average, the one that admits all 512 included,
+// and the burst 3.9 ms instead of 5.7.  The pinned per-call buffers rotate, each
+// reused only after the call that last used it has finished on the device, which
+// also bounds how far the host runs ahead.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <deque>
+#include <functional>
 #include <string>
 #include <vector>
 
-#include "snn_internal.cuh"
 #include "snn_nvtx.cuh"
+#include "snn_sample.cuh"
 
 namespace snn {
 const snn_spec& net_spec(const snn_net* n);
@@ -63,27 +70,20 @@ struct SlotBufs {
     uint32_t* cnt;         // [S] inhibitory spikes of the slot's previous step
     int* t_loc;            // [S] steps taken by the slot's request
     int* t_len;            // [S] its presentation length
-    uint32_t* ring;        // [R][N] result rows
+    uint32_t* ring;        // [R][N] result rows (pinned host memory)
 };
 
-// Device side of one call's host staging.
-struct CallBufs {
-    float* rates;          // [S][n_in] admitted rates
-    int* adm;              // [S] admitted slots
-    int* adm_len;          // [S] their lengths
-    uint64_t* adm_seed;    // [S] their seeds
-    int* live;             // [S] slots that step in this call
-    int* fin;              // [S] slots retired by this call
-    int* fin_row;          // [S] their result rows
-};
+// One call's lists, in pinned host memory that the kernels read.
+struct Admission { int slot, len; uint64_t seed; };
+struct Live { int slot, row; };         // a slot that steps; its result row if it ends in the call, else -1
 
 // Admitted slot a: thresholds from its rates, state reset, counters.
-__global__ void k_serve_admit(snn::Consts c, SlotBufs d, CallBufs cb, int n_adm) {
+__global__ void k_serve_admit(snn::Consts c, SlotBufs d, const Admission* adm, const float* rates) {
     const int a = blockIdx.x;
-    if (a >= n_adm) return;
-    const int s = cb.adm[a];
+    const Admission ad = adm[a];
+    const int s = ad.slot;
     for (int i = threadIdx.x; i < c.n_in; i += blockDim.x)
-        d.thr[(size_t)s * c.n_in + i] = snn::poisson_threshold(cb.rates[(size_t)a * c.n_in + i], c.dt);
+        d.thr[(size_t)s * c.n_in + i] = snn::poisson_threshold(rates[(size_t)a * c.n_in + i], c.dt);
     for (int j = threadIdx.x; j < c.N; j += blockDim.x) {
         const size_t k = (size_t)s * c.N + j;
         d.v_e[k] = c.e_rest;
@@ -93,24 +93,55 @@ __global__ void k_serve_admit(snn::Consts c, SlotBufs d, CallBufs cb, int n_adm)
     }
     if (threadIdx.x == 0) {
         d.cnt[s] = 0u;
-        d.seeds[s] = cb.adm_seed[a];
+        d.seeds[s] = ad.seed;
         d.t_loc[s] = 0;
-        d.t_len[s] = cb.adm_len[a];
+        d.t_len[s] = ad.len;
     }
 }
 
-// One CTA per live slot runs up to k of its steps: the input spikes of the
-// step, the ascending list of active inputs, and snn_run's neuron update for
-// each of the slot's neurons (current summed over the list in ascending
-// order), the inhibitory count of the step kept in the CTA for the next.
-__global__ void __launch_bounds__(SC_THREADS) k_serve_chunk(snn::Consts c, SlotBufs d, const int* __restrict__ live,
-                                                            int k) {
+// One CTA per live slot runs up to k of its steps (snn_sample.cuh), the state
+// in registers between them.
+template <int NPT>
+__global__ void __launch_bounds__(1024, 1) k_serve_chunk(const __grid_constant__ snn::Consts c,
+                                                         const __grid_constant__ SlotBufs d,
+                                                         const Live* __restrict__ live, int k) {
+    extern __shared__ __align__(16) unsigned char ssm[];
+    const Live lv = live[blockIdx.x];
+    const int s = lv.slot;
+    const int t0 = d.t_loc[s];
+    const int steps = min(k, d.t_len[s] - t0);
+    if (steps <= 0) return;                             // (uniform over the CTA)
+    const size_t sn = (size_t)s * c.N;
+    snn::SampleIO io{};
+    io.W = d.W;
+    io.theta = d.theta;
+    io.wscale = d.wscale;
+    io.thr = d.thr + (size_t)s * c.n_in;
+    io.seed = d.seeds[s];
+    io.v_e = d.v_e + sn;
+    io.v_i = d.v_i + sn;
+    io.st = d.st + sn;
+    io.counts = d.counts + sn;
+    const int C = snn::run_sample<NPT, false>(c, io, (unsigned long long)t0, steps, (int)d.cnt[s], ssm);
+    if (lv.row >= 0)                                    // (each thread's own counts)
+        for (int j = threadIdx.x; j < c.N; j += blockDim.x) d.ring[(size_t)lv.row * c.N + j] = io.counts[j];
+    if (threadIdx.x == 0) {
+        d.t_loc[s] = t0 + steps;
+        d.cnt[s] = (uint32_t)C;
+    }
+}
+
+// Layers too wide for a thread's registers: the same step with the state in
+// global memory, a loop over the neurons.
+__global__ void __launch_bounds__(SC_THREADS) k_serve_chunk_wide(snn::Consts c, SlotBufs d,
+                                                                 const Live* __restrict__ live, int k) {
     extern __shared__ uint32_t sh[];
     uint32_t* words = sh;                               // [Iw] input spike words of the step
     uint16_t* act = (uint16_t*)(sh + c.Iw);             // [n_in] active inputs, ascending
     __shared__ int s_nact;
     __shared__ uint32_t s_cnt[2];
-    const int s = live[blockIdx.x];
+    const Live lv = live[blockIdx.x];
+    const int s = lv.slot;
     const int t0 = d.t_loc[s];
     const int steps = min(k, d.t_len[s] - t0);
     if (steps <= 0) return;                             // (uniform over the CTA)
@@ -182,19 +213,12 @@ __global__ void __launch_bounds__(SC_THREADS) k_serve_chunk(snn::Consts c, SlotB
         __syncthreads();
         C = (int)s_cnt[t & 1];
     }
+    if (lv.row >= 0)                                    // (each thread's own counts)
+        for (int j = threadIdx.x; j < c.N; j += blockDim.x) d.ring[(size_t)lv.row * c.N + j] = d.counts[(size_t)s * c.N + j];
     if (threadIdx.x == 0) {
         d.t_loc[s] = t0 + steps;
         d.cnt[s] = (uint32_t)C;
     }
-}
-
-// The retired slots' spike counts into their result rows.
-__global__ void k_serve_gather(snn::Consts c, SlotBufs d, CallBufs cb, int n_fin) {
-    const int f = blockIdx.x;
-    if (f >= n_fin) return;
-    const int s = cb.fin[f];
-    uint32_t* row = d.ring + (size_t)cb.fin_row[f] * c.N;
-    for (int j = threadIdx.x; j < c.N; j += blockDim.x) row[j] = d.counts[(size_t)s * c.N + j];
 }
 
 __global__ void k_serve_scales(snn::Consts c, SlotBufs d) {
@@ -229,25 +253,20 @@ struct Pending {
     std::vector<int> rows;
 };
 
-// Host staging of one call (pinned) and its device counterpart.
+// One call's pinned buffers.
 struct Stage {
-    float* rates = nullptr;
-    int* adm = nullptr;
-    int* adm_len = nullptr;
-    uint64_t* adm_seed = nullptr;
-    int* live = nullptr;
-    int* fin = nullptr;
-    int* fin_row = nullptr;
-    CallBufs dev{};
+    float* rates = nullptr;       // [S][n_in] admitted rates
+    Admission* adm = nullptr;     // [S]
+    Live* live = nullptr;         // [S]
     cudaEvent_t done = nullptr;   // the call that last used this stage has finished
     bool used = false;
 };
 
 size_t slot_bytes_of(const snn_spec& sp) {
     const size_t NI = sp.n_in, N = sp.n_exc;
-    // device: thresholds, seed, voltages, packed refractory/spike word, counts,
-    // the inhibitory count and step counters, two result rows, and one slot's
-    // share of each call's staging (rates, slot lists) in every stage
+    // thresholds, seed, voltages, packed refractory/spike word, counts, the
+    // inhibitory count and step counters on the device; two result rows and one
+    // slot's share of each call's lists (rates, slots) in every stage, pinned
     return NI * 4 + 8 + N * 16 + 12 + 2 * N * 4 + STAGES * (NI * 4 + 4 * 7);
 }
 
@@ -264,8 +283,10 @@ struct snn_server {
     std::vector<void*> host_allocs;
     Stage stage[STAGES];
     int next_stage = 0;
-    uint32_t* h_ring = nullptr;    // pinned [R][N]
     std::vector<int> free_rows;
+    std::vector<int> free_slots;   // a heap, the lowest first
+    std::vector<int> active;       // slots with steps left, ascending
+    std::vector<cudaEvent_t> free_events;
     std::deque<Request> queue;
     std::vector<Slot> slots;
     std::deque<Pending> pending;
@@ -318,12 +339,12 @@ cudaError_t collect(snn_server* s, bool wait_oldest) {
         for (size_t f = 0; f < p.ids.size(); ++f) {
             Result r;
             r.id = p.ids[f];
-            const uint32_t* row = s->h_ring + (size_t)p.rows[f] * N;
+            const uint32_t* row = s->d.ring + (size_t)p.rows[f] * N;
             r.counts.assign(row, row + N);
             s->done.push_back(std::move(r));
             s->free_rows.push_back(p.rows[f]);
         }
-        cudaEventDestroy(p.ev);
+        s->free_events.push_back(p.ev);
         s->pending.pop_front();
     }
     return cudaSuccess;
@@ -342,6 +363,7 @@ snn_status snn_serve_destroy(snn_server* s) {
     cudaSetDevice(s->device);
     cudaDeviceSynchronize();
     for (Pending& p : s->pending) if (p.ev) cudaEventDestroy(p.ev);
+    for (cudaEvent_t e : s->free_events) cudaEventDestroy(e);
     for (Stage& st : s->stage) if (st.done) cudaEventDestroy(st.done);
     for (void* p : s->allocs) cudaFree(p);
     for (void* p : s->host_allocs) cudaFreeHost(p);
@@ -389,27 +411,16 @@ snn_status snn_serve_create(snn_net* net, int max_slots, size_t state_cap_bytes,
     if (e == cudaSuccess) e = salloc(s, &d.cnt, (size_t)S);
     if (e == cudaSuccess) e = salloc(s, &d.t_loc, (size_t)S);
     if (e == cudaSuccess) e = salloc(s, &d.t_len, (size_t)S);
-    if (e == cudaSuccess) e = salloc(s, &d.ring, (size_t)s->R * N);
-    if (e == cudaSuccess) e = halloc(s, &s->h_ring, (size_t)s->R * N);
+    if (e == cudaSuccess) e = halloc(s, &d.ring, (size_t)s->R * N);
     for (int k = 0; k < STAGES && e == cudaSuccess; ++k) {
         Stage& st = s->stage[k];
         e = halloc(s, &st.rates, (size_t)S * NI);
         if (e == cudaSuccess) e = halloc(s, &st.adm, (size_t)S);
-        if (e == cudaSuccess) e = halloc(s, &st.adm_len, (size_t)S);
-        if (e == cudaSuccess) e = halloc(s, &st.adm_seed, (size_t)S);
         if (e == cudaSuccess) e = halloc(s, &st.live, (size_t)S);
-        if (e == cudaSuccess) e = halloc(s, &st.fin, (size_t)S);
-        if (e == cudaSuccess) e = halloc(s, &st.fin_row, (size_t)S);
-        if (e == cudaSuccess) e = salloc(s, &st.dev.rates, (size_t)S * NI);
-        if (e == cudaSuccess) e = salloc(s, &st.dev.adm, (size_t)S);
-        if (e == cudaSuccess) e = salloc(s, &st.dev.adm_len, (size_t)S);
-        if (e == cudaSuccess) e = salloc(s, &st.dev.adm_seed, (size_t)S);
-        if (e == cudaSuccess) e = salloc(s, &st.dev.live, (size_t)S);
-        if (e == cudaSuccess) e = salloc(s, &st.dev.fin, (size_t)S);
-        if (e == cudaSuccess) e = salloc(s, &st.dev.fin_row, (size_t)S);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&st.done, cudaEventDisableTiming);
     }
     for (int r = s->R - 1; r >= 0; --r) s->free_rows.push_back(r);
+    for (int k = 0; k < S; ++k) s->free_slots.push_back(k);   // ascending: a heap, the lowest first
     if (e == cudaSuccess) e = cudaMemset(d.t_len, 0, (size_t)S * 4);
     if (e == cudaSuccess) e = cudaMemset(d.t_loc, 0, (size_t)S * 4);
     if (e == cudaSuccess && sp.wprec == SNN_W_FP8E4M3) {   // the frozen W's column scales
@@ -453,83 +464,85 @@ snn_status snn_serve_step(snn_server* s, int k, void* stream_, int* steps_run) {
     if (steps_run) *steps_run = 0;
     cudaStream_t st = (cudaStream_t)stream_;
     SERVE_CUDA(s, cudaSetDevice(s->device));
-    const int S = s->S, NI = s->c.n_in, N = s->c.N;
-    // this call's staging: free once the call that used it last has finished
+    const int NI = s->c.n_in, N = s->c.N;
+    // this call's buffers: free once the call that used them last has finished
     Stage& sg = s->stage[s->next_stage];
     s->next_stage = (s->next_stage + 1) % STAGES;
     if (sg.used) SERVE_CUDA(s, cudaEventSynchronize(sg.done));
     SERVE_CUDA(s, collect(s, false));
-    // ---- admit queued requests into free slots
+    // ---- admit queued requests into free slots, the lowest first
     int na = 0;
-    for (int slot = 0; slot < S && !s->queue.empty(); ++slot) {
-        if (s->slots[slot].remaining > 0) continue;
+    const size_t before = s->active.size();
+    while (!s->free_slots.empty() && !s->queue.empty()) {
+        std::pop_heap(s->free_slots.begin(), s->free_slots.end(), std::greater<int>());
+        const int slot = s->free_slots.back();
+        s->free_slots.pop_back();
         Request& r = s->queue.front();
         std::memcpy(sg.rates + (size_t)na * NI, r.rates.data(), (size_t)NI * 4);
-        sg.adm[na] = slot;
-        sg.adm_len[na] = r.T;
-        sg.adm_seed[na] = r.seed;
+        sg.adm[na] = Admission{slot, r.T, r.seed};
         s->slots[slot].id = r.id;
         s->slots[slot].remaining = r.T;
+        s->active.push_back(slot);
         s->queue.pop_front();
         ++na;
     }
+    std::inplace_merge(s->active.begin(), s->active.begin() + before, s->active.end());
     if (na > 0) {
-        SERVE_CUDA(s, cudaMemcpyAsync(sg.dev.rates, sg.rates, (size_t)na * NI * 4, cudaMemcpyHostToDevice, st));
-        SERVE_CUDA(s, cudaMemcpyAsync(sg.dev.adm, sg.adm, (size_t)na * 4, cudaMemcpyHostToDevice, st));
-        SERVE_CUDA(s, cudaMemcpyAsync(sg.dev.adm_len, sg.adm_len, (size_t)na * 4, cudaMemcpyHostToDevice, st));
-        SERVE_CUDA(s, cudaMemcpyAsync(sg.dev.adm_seed, sg.adm_seed, (size_t)na * 8, cudaMemcpyHostToDevice, st));
-        k_serve_admit<<<na, 256, 0, st>>>(s->c, s->d, sg.dev, na);
+        k_serve_admit<<<na, 256, 0, st>>>(s->c, s->d, sg.adm, sg.rates);
         SERVE_CUDA(s, cudaGetLastError());
     }
-    // ---- up to k steps of every live slot, one CTA per slot
-    int nl = 0, longest = 0;
-    for (int slot = 0; slot < S; ++slot)
-        if (s->slots[slot].remaining > 0) {
-            sg.live[nl++] = slot;
-            longest = s->slots[slot].remaining > longest ? s->slots[slot].remaining : longest;
-        }
+    // ---- up to k steps of every live slot, one CTA per slot; those that end
+    // within them are retired, each with a result row
+    int longest = 0, nf = 0;
+    for (int slot : s->active) longest = s->slots[slot].remaining > longest ? s->slots[slot].remaining : longest;
     const int kk = k < longest ? k : longest;
+    for (int slot : s->active) nf += s->slots[slot].remaining <= kk;
+    while ((int)s->free_rows.size() < nf) {               // the ring is full: wait for the oldest batch
+        if (s->pending.empty()) return sfail(s, SNN_ERR_CUDA, "snn_serve_step: result ring exhausted");
+        SERVE_CUDA(s, collect(s, true));
+    }
+    Pending p;
+    int nl = 0, left = 0;
+    for (int slot : s->active) {
+        Slot& sl = s->slots[slot];
+        sl.remaining -= kk;
+        Live& lv = sg.live[nl++];
+        lv = Live{slot, -1};
+        if (sl.remaining > 0) {
+            s->active[left++] = slot;
+            continue;
+        }
+        sl.remaining = 0;
+        lv.row = s->free_rows.back();
+        s->free_rows.pop_back();
+        p.ids.push_back(sl.id);
+        p.rows.push_back(lv.row);
+        s->free_slots.push_back(slot);
+        std::push_heap(s->free_slots.begin(), s->free_slots.end(), std::greater<int>());
+    }
+    s->active.resize(left);
     if (nl > 0) {
-        SERVE_CUDA(s, cudaMemcpyAsync(sg.dev.live, sg.live, (size_t)nl * 4, cudaMemcpyHostToDevice, st));
-        const size_t smem = (size_t)s->c.Iw * 4 + (size_t)NI * 2 + 16;
-        k_serve_chunk<<<nl, SC_THREADS, smem, st>>>(s->c, s->d, sg.dev.live, kk);
+        const int npt = NI <= 65535 ? snn::sample_npt(N) : 0;
+        const size_t need = snn::sample_smem(NI, s->c.Iw, false, false).bytes;
+        if (npt == 0 || need > 48 * 1024) {
+            const size_t smem = (size_t)s->c.Iw * 4 + (size_t)NI * 2 + 16;
+            k_serve_chunk_wide<<<nl, SC_THREADS, smem, st>>>(s->c, s->d, sg.live, kk);
+        } else {
+            auto kern = npt == 1 ? k_serve_chunk<1> : npt == 2 ? k_serve_chunk<2>
+                      : npt == 4 ? k_serve_chunk<4> : k_serve_chunk<8>;
+            kern<<<nl, snn::sample_threads(N, npt), need, st>>>(s->c, s->d, sg.live, kk);
+        }
         SERVE_CUDA(s, cudaGetLastError());
     }
     if (steps_run) *steps_run = kk;
-    // ---- retire the slots whose presentation ended, their counts into result rows
-    int nf = 0;
-    std::vector<uint64_t> ids;
-    for (int slot = 0; slot < S; ++slot) {
-        Slot& sl = s->slots[slot];
-        if (sl.remaining <= 0) continue;
-        sl.remaining -= kk;
-        if (sl.remaining <= 0) {
-            sl.remaining = 0;
-            sg.fin[nf++] = slot;
-            ids.push_back(sl.id);
-        }
-    }
     if (nf > 0) {
-        while ((int)s->free_rows.size() < nf) {           // the ring is full: wait for the oldest batch
-            if (s->pending.empty()) return sfail(s, SNN_ERR_CUDA, "snn_serve_step: result ring exhausted");
-            SERVE_CUDA(s, collect(s, true));
+        if (s->free_events.empty()) {
+            SERVE_CUDA(s, cudaEventCreateWithFlags(&p.ev, cudaEventDisableTiming));
+        } else {
+            p.ev = s->free_events.back();
+            s->free_events.pop_back();
         }
-        Pending p;
-        for (int f = 0; f < nf; ++f) {
-            sg.fin_row[f] = s->free_rows.back();
-            s->free_rows.pop_back();
-            p.rows.push_back(sg.fin_row[f]);
-        }
-        SERVE_CUDA(s, cudaMemcpyAsync(sg.dev.fin, sg.fin, (size_t)nf * 4, cudaMemcpyHostToDevice, st));
-        SERVE_CUDA(s, cudaMemcpyAsync(sg.dev.fin_row, sg.fin_row, (size_t)nf * 4, cudaMemcpyHostToDevice, st));
-        k_serve_gather<<<nf, 256, 0, st>>>(s->c, s->d, sg.dev, nf);
-        SERVE_CUDA(s, cudaGetLastError());
-        for (int f = 0; f < nf; ++f)                       // rows are not contiguous: one copy each
-            SERVE_CUDA(s, cudaMemcpyAsync(s->h_ring + (size_t)p.rows[f] * N, s->d.ring + (size_t)p.rows[f] * N,
-                                          (size_t)N * 4, cudaMemcpyDeviceToHost, st));
-        SERVE_CUDA(s, cudaEventCreateWithFlags(&p.ev, cudaEventDisableTiming));
         SERVE_CUDA(s, cudaEventRecord(p.ev, st));
-        p.ids = std::move(ids);
         s->pending.push_back(std::move(p));
     }
     SERVE_CUDA(s, cudaEventRecord(sg.done, st));
@@ -565,8 +578,7 @@ snn_status snn_serve_wait(snn_server* s) {
 
 snn_status snn_serve_status(const snn_server* s, int* slots, int* active, int* queued, int* done) {
     if (!s) return SNN_ERR_ARG;
-    int a = 0;
-    for (const Slot& sl : s->slots) a += sl.remaining > 0;
+    const int a = (int)s->active.size();
     size_t in_flight = 0;
     for (const Pending& p : s->pending) in_flight += p.ids.size();
     if (slots) *slots = s->S;
