@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(32 * (GNW_MAX + GE), 1) k_rec_gather(RecConsts
 #pragma unroll
                 for (int q = 0; q < GR; ++q)
                     src[q] = wsrc + (size_t)((ii[q >> 1] >> (16 * (q & 1))) & 0xFFFFu) * wpitch;
-                if (i >= g.S && ok) ok = mbar_wait(&empty[s], ((i >> g.lgS) - 1) & 1);
+                if (i >= g.S && ok) ok = snn::tc::mbar_wait_short(&empty[s], ((i >> g.lgS) - 1) & 1, GWAIT_NS);
                 ok = __all_sync(FULL, ok ? 1 : 0) != 0;
                 if (!ok) break;
                 for (int x = 16 * lane; x < cb; x += 512)
@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(32 * (GNW_MAX + GE), 1) k_rec_gather(RecConsts
             for (int q = 0; q < VEC; ++q) x[q] = 0.0f;
             for (int k = 0; k < nst && cb > 0; ++k) {
                 const int i = it + k, s = i & (g.S - 1);
-                if (ok) ok = mbar_wait(&full[s], (i >> g.lgS) & 1);
+                if (ok) ok = snn::tc::mbar_wait_short(&full[s], (i >> g.lgS) & 1, GWAIT_NS);
                 const uint8_t* src = gsm + s * GR * RB + tid * (VEC * 2);
                 constexpr int U = VEC == 8 ? 4 : GR;       // rows loaded together (registers)
 #pragma unroll
@@ -1222,10 +1222,12 @@ snn_status snn_rec_create(const snn_rec_spec* spec, snn_rec** out) {
         if (e == cudaSuccess) e = cudaMemset(r->w_ff + (nw - ldw), 0, ldw * 2);
         if (e == cudaSuccess) e = cudaMemcpy(r->w_ff, s.w_ff, s.n_in * row, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(r->w_rec, s.w_rec, s.n_hid * row, cudaMemcpyHostToDevice);
-    } else {
+    } else {   // padded on the device, from the stacked operand's memory (at least as large, packed below)
         if (e == cudaSuccess) e = cudaMemset(r->w_ff, 0, nw * 2);
-        if (e == cudaSuccess) e = cudaMemcpy2D(r->w_ff, ldw * 2, s.w_ff, row, row, s.n_in, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy2D(r->w_rec, ldw * 2, s.w_rec, row, row, s.n_hid, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(r->wt, s.w_ff, s.n_in * row, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(r->wt + (size_t)s.n_in * s.n_hid, s.w_rec, s.n_hid * row, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess)
+            e = cudaMemcpy2D(r->w_ff, ldw * 2, r->wt, row, row, (size_t)s.n_in + s.n_hid, cudaMemcpyDeviceToDevice);
     }
     if (e == cudaSuccess) e = cudaMemset(r->w_out + nout, 0, (size_t)s.n_out * 2);
     if (e == cudaSuccess) e = cudaMemcpy(r->w_out, s.w_out, nout * 2, cudaMemcpyHostToDevice);
