@@ -35,6 +35,8 @@ namespace snn {
 
 // The learning-off form (snn_infer.cu); *used = 0 where it does not apply.
 cudaError_t launch_infer(const Consts& c, const Bufs& d, int T, cudaStream_t s, int* used);
+// The small-batch learning form (snn_small.cu), likewise.
+cudaError_t launch_small(const Consts& c, const Bufs& d, int T, cudaStream_t s, int* used);
 
 namespace {
 
@@ -1921,10 +1923,11 @@ cudaError_t launch_persistent(const Consts& c, const Bufs& d, int T, cudaStream_
         attr = L.bytes;
     }
     lock.unlock();
-    if (!c.learn) {   // nothing couples the samples: a CTA per sample
+    {   // learning off: nothing couples the samples, a CTA per sample; few samples:
+        // the network in one cluster
         e = prof_start(prof, SNN_KERNEL_PERSISTENT, s);
         if (e != cudaSuccess) return e;
-        e = launch_infer(c, d, T, s, used);
+        e = c.learn ? launch_small(c, d, T, s, used) : launch_infer(c, d, T, s, used);
         if (e != cudaSuccess) return e;
         if (*used) return prof_stop(prof, s);
         if (prof) prof->n -= 1;               // not taken: the event is recorded again below

@@ -87,3 +87,27 @@ def test_learning_off_sample_per_cta(B, NI, N, T, wprec):
     net, g = tp.gpu_run(p, r, s, w, 4, mode="graph", net=net, continue_=True)
     tp.assert_parity(g, st, rec)
     net.close()
+
+
+@pytest.mark.parametrize("B,NI,N,T,reduce,wprec", [
+    (1, 784, 100, 120, "max", 0),      # every sample an event; CTAs of 13 columns, the last short
+    (1, 40, 5, 150, "mean", 0),        # fewer columns than CTAs
+    (5, 1100, 500, 60, "sum", 1),      # 35 input words, 32 columns a CTA
+    (4, 300, 1700, 40, "mean", 0),     # 107 columns: four column rounds, two items a thread
+    (11, 300, 620, 60, "mean", 0),     # 39 columns: two column rounds
+    (32, 100, 200, 60, "max", 0),      # full masks
+])
+def test_small_batch_cluster(B, NI, N, T, reduce, wprec):
+    """The small-batch learning form, and what it leaves: a continuing run with
+    other rates (traces of inputs that no longer spike), then the graph form."""
+    import test_gpu_parity as tp
+    p, r, s, w = tp.synth.workload(B, N, NI)
+    r = np.minimum(r * np.float32(4 * 784 / NI), np.float32(900))       # the oracle fires in every case
+    r2 = np.roll(r, 5, axis=1)
+    net, st = None, None
+    for k, (rates, steps, mode) in enumerate([(r, T, "persistent"), (r2, 30, "persistent"), (r, 10, "graph")]):
+        st, rec = tp.oracle_run(p, rates, s, w, steps, reduce=reduce, st=st, episodic=k == 0, wprec=wprec)
+        net, g = tp.gpu_run(p, rates, s, w, steps, reduce=reduce, mode=mode, net=net, continue_=k > 0, wprec=wprec)
+        tp.assert_parity(g, st, rec)
+        assert k > 0 or rec.raster_e.sum() > 0
+    net.close()
