@@ -91,6 +91,7 @@ struct RecBufs {
     uint64_t* seeds;         // [B]
     uint32_t* inb;           // [B][Iw]     input spikes of the step
     uint32_t* sh;            // [2][B][Nw]  hidden spikes, slot = step parity
+    uint32_t* hist;          // [HIST][Bp/32][Nw][32] the tensor form's spike words not yet in the counts
     float* v;                // [Bp/32][N][32], Bp = B rounded up to 32 (sidx)
     float* i_syn;            // [Bp/32][N][32]
     float* v_out;            // [B][n_out]
@@ -123,9 +124,13 @@ static_assert(GBM == 128, "the instruction descriptor is for M = 128");
 // weight rows start at R0 = ntn_drive * GBN and whose MMAs are n_ro wide.
 // With enc_next, drive tile (tm, tn) also draws the next step's input spikes of
 // its samples for inputs [tn * a_per, (tn + 1) * a_per), a_per a multiple of 32.
+// Every step's spike words go to hist slot `slot`; to sh only with keep_sh (the
+// run's last step, or a readout launch of its own).
 struct DenseGeom {
     int ntn_drive, ntn, ntiles, fused, n_ro, a_per, enc_next;
+    int slot, keep_sh;
 };
+constexpr int HIST = 31;                 // steps between two updates of the counts (five-bit counters)
 
 // waits for the phase with the given parity to complete; false after GWAIT_NS
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity) {
@@ -633,17 +638,52 @@ __device__ __forceinline__ void dense_encode_group(const RecConsts& c, const Rec
     store_operand_word(c, d, b, live, word, (int)(tt & 1ull), a0, nu);
 }
 
+// the spike word of neurons 32 jw .. of sample b
+__device__ __forceinline__ void keep_word(const RecConsts& c, const RecBufs& d, const DenseGeom& g, int b, int jw,
+                                          int cur, uint32_t word) {
+    const size_t bp = (size_t)((c.B + 31) >> 5);
+    d.hist[(((size_t)g.slot * bp + (b >> 5)) * c.Nw + jw) * 32 + (b & 31)] = word;
+    if (g.keep_sh) d.sh[((size_t)cur * c.B + b) * c.Nw + jw] = word;
+}
+
+// counts += the spikes of hist slots 0 .. n - 1: lane = sample, warp = a word of
+// 32 neurons; the words are summed bit by bit in five counter words, so the
+// counts are read and written once for n steps (in the epilogue they were a third
+// of its state bytes, every step).
+__global__ void __launch_bounds__(256) k_rec_fold(RecConsts c, RecBufs d, int n) {
+    const int lane = threadIdx.x & 31;
+    const size_t gw = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const size_t bp = (size_t)((c.B + 31) >> 5);
+    if (gw >= bp * c.Nw) return;
+    const int b = (int)(gw / c.Nw) * 32 + lane, jw = (int)(gw % c.Nw);
+    if (b >= c.B) return;
+    uint32_t k0 = 0u, k1 = 0u, k2 = 0u, k3 = 0u, k4 = 0u;
+#pragma unroll 8
+    for (int s = 0; s < n; ++s) {
+        uint32_t x = d.hist[((size_t)s * bp * c.Nw + gw) * 32 + lane], t;
+        t = k0 & x; k0 ^= x; x = t;
+        t = k1 & x; k1 ^= x; x = t;
+        t = k2 & x; k2 ^= x; x = t;
+        t = k3 & x; k3 ^= x; x = t;
+        k4 ^= x;
+    }
+    uint32_t* p = d.counts + sidx(b, jw * 32, c.N);
+    const int nu = min(32, c.N - jw * 32);
+#pragma unroll 8
+    for (int u = 0; u < nu; ++u)
+        p[32 * u] += ((k0 >> u) & 1u) | ((k1 >> u) & 1u) << 1 | ((k2 >> u) & 1u) << 2 | ((k3 >> u) & 1u) << 3 |
+                     ((k4 >> u) & 1u) << 4;
+}
+
 // Dense form, epilogue of one warp's half tile (32 samples x 128 neurons j0..,
-// all < N) as a 2-deep pipeline over 16-neuron steps: the state loads of step
-// k+1 are in flight while step k is computed and stored, so the loads of
-// consecutive steps leave no gap.  (A third slot would not fit the 168
-// registers a thread has at this block size.)  The warp's accumulator is
+// all < N) as a 3-deep pipeline over 16-neuron steps: the state loads of steps
+// k+1 and k+2 are in flight while step k is computed and stored, so the loads of
+// consecutive steps leave no gap.  The warp's accumulator is
 // released (acce) after its last tensor-memory load.  Each pipeline slot is a
 // template argument, so every register index is a compile-time constant.
-constexpr int EPD = 2, EPH = 8;   // pipeline depth, 16-neuron steps per half tile
+constexpr int EPD = 3, EPH = 8;   // pipeline depth, 16-neuron steps per half tile
 struct EpiSlot {
     float I[16], V[16];
-    uint32_t CN[16];
 };
 
 __device__ __forceinline__ void epi_load(const RecConsts& c, const RecBufs& d, EpiSlot& sl, int b, int j) {
@@ -652,14 +692,13 @@ __device__ __forceinline__ void epi_load(const RecConsts& c, const RecBufs& d, E
     for (int u = 0; u < 16; ++u) {
         sl.I[u] = d.i_syn[q0 + 32 * u];
         sl.V[u] = d.v[q0 + 32 * u];
-        sl.CN[u] = d.counts[q0 + 32 * u];
     }
 }
 
 template <int K>
 __device__ __forceinline__ void epi_step(const RecConsts& c, const RecBufs& d, const EpiSlot& sl, uint32_t tcol,
                                          int b, bool live, int j0, int cur, int nxt, int t_local,
-                                         uint64_t* acce_bar, uint32_t& word) {
+                                         uint64_t* acce_bar, const DenseGeom& g, uint32_t& word) {
     const int lane = threadIdx.x & 31;
     uint32_t r[16];
     tmem_ld16(tcol + (uint32_t)(16 * K), r);
@@ -680,7 +719,6 @@ __device__ __forceinline__ void epi_step(const RecConsts& c, const RecBufs& d, c
             const bool spk = y >= c.v_thresh;
             d.i_syn[q0 + 32 * u] = x;
             d.v[q0 + 32 * u] = spk ? c.v_reset : y;
-            d.counts[q0 + 32 * u] = sl.CN[u] + (spk ? 1u : 0u);
             w16 |= (spk ? 1u : 0u) << u;
         }
         if (c.rec_raster) {
@@ -691,7 +729,7 @@ __device__ __forceinline__ void epi_step(const RecConsts& c, const RecBufs& d, c
     word |= w16 << (16 * (K & 1));
     if (K & 1) {                                          // a full 32-neuron word
         const int jw0 = j0 + 16 * (K - 1);
-        if (live) d.sh[((size_t)cur * c.B + b) * c.Nw + (jw0 >> 5)] = word;
+        if (live) keep_word(c, d, g, b, jw0 >> 5, cur, word);
         store_operand_word(c, d, b, live, word, nxt, c.n_in + jw0, 32);
         word = 0u;
     }
@@ -701,28 +739,29 @@ __device__ __forceinline__ void epi_step(const RecConsts& c, const RecBufs& d, c
 template <int H>
 __device__ __forceinline__ void epi_iter(const RecConsts& c, const RecBufs& d, EpiSlot (&sl)[EPD], uint32_t tcol,
                                          int b, bool live, int j0, int cur, int nxt, int t_local,
-                                         uint64_t* acce_bar, uint32_t& word) {
+                                         uint64_t* acce_bar, const DenseGeom& g, uint32_t& word) {
     if (H < EPH && live) epi_load(c, d, sl[H % EPD], b, j0 + 16 * H);
     if (H >= EPD - 1)
         epi_step<(H >= EPD - 1 ? H - (EPD - 1) : 0)>(c, d, sl[(H >= EPD - 1 ? H - (EPD - 1) : 0) % EPD], tcol, b, live,
-                                                     j0, cur, nxt, t_local, acce_bar, word);
+                                                     j0, cur, nxt, t_local, acce_bar, g, word);
 }
 
 __device__ __forceinline__ void dense_epilogue_half_pipelined(const RecConsts& c, const RecBufs& d, uint32_t tcol,
                                                               int b, bool live, int j0, int cur, int nxt,
-                                                              int t_local, uint64_t* acce_bar) {
-    static_assert(EPD == 2 && EPH == 8, "the iterations below are written out for these sizes");
+                                                              int t_local, uint64_t* acce_bar, const DenseGeom& g) {
+    static_assert(EPD == 3 && EPH == 8, "the iterations below are written out for these sizes");
     EpiSlot sl[EPD];
     uint32_t word = 0u;
-    epi_iter<0>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, word);
-    epi_iter<1>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, word);
-    epi_iter<2>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, word);
-    epi_iter<3>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, word);
-    epi_iter<4>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, word);
-    epi_iter<5>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, word);
-    epi_iter<6>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, word);
-    epi_iter<7>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, word);
-    epi_iter<8>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, word);
+    epi_iter<0>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<1>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<2>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<3>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<4>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<5>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<6>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<7>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<8>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<9>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
 }
 
 // Dense form, persistent: one CTA per SM walks the 128-sample x 256-neuron
@@ -840,7 +879,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
             const bool piped = !ro && (half + 1) * CH * 32 <= ncols && (c.n_in & 1) == 0;
             if (piped)
                 dense_epilogue_half_pipelined(c, d, tbase + (uint32_t)(half * CH * 32), b, b < c.B,
-                                              tn * GBN + half * CH * 32, cur, nxt, t_local, &acce[buf]);
+                                              tn * GBN + half * CH * 32, cur, nxt, t_local, &acce[buf], g);
             // otherwise (a half tile past the layer's end, or the readout tile):
             // 16-column steps, each neuron guarded
             uint32_t word = 0u;
@@ -870,8 +909,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
                             y = __fadd_rn(y, x);
                             const bool spk = y >= c.v_thresh;
                             d.v[qq] = spk ? c.v_reset : y;
-                            if (spk) d.counts[qq] += 1u;
-                            w16 |= (spk ? 1u : 0u) << u;
+                                            w16 |= (spk ? 1u : 0u) << u;
                         }
                         if (c.rec_raster) {
                             uint8_t* rp = d.raster_h + ((size_t)t_local * c.B + b) * c.N + j;
@@ -881,7 +919,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
                     word |= w16 << (16 * (q & 1));
                     if ((q & 1) || col + 16 >= ncols) {     // the 32-neuron word is complete
                         const int jw0 = j - 16 * (q & 1), nu32 = min(32, c.N - jw0);
-                        if (b < c.B) d.sh[((size_t)cur * c.B + b) * c.Nw + (jw0 >> 5)] = word;
+                        if (b < c.B) keep_word(c, d, g, b, jw0 >> 5, cur, word);
                         store_operand_word(c, d, b, b < c.B, word, nxt, c.n_in + jw0, nu32);
                         word = 0u;
                     }
@@ -1103,7 +1141,7 @@ snn_status rec_fail(snn_rec* r, snn_status code, const char* fmt, ...) {
 
 void free_batch(snn_rec* r) {
     void* ptrs[] = {r->d.thr, r->d.seeds, r->d.inb, r->d.sh, r->d.v, r->d.i_syn, r->d.v_out,
-                    r->d.counts, r->d.raster_h, r->d.raster_in, r->rates_stage, r->seeds_stage, r->d.S};
+                    r->d.counts, r->d.hist, r->d.raster_h, r->d.raster_in, r->rates_stage, r->seeds_stage, r->d.S};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     const RecBufs keep = r->d;
@@ -1335,6 +1373,10 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
         form = (r->activity >= 0.0 && r->activity < cut) ? SNN_REC_GATHER : SNN_REC_TENSOR;
     }
     const int dense = form == SNN_REC_TENSOR ? 1 : 0;
+    if (dense && !r->d.hist) {
+        if (r->last) REC_TRY(r, cudaStreamSynchronize(r->last));
+        REC_TRY(r, dalloc(&r->d.hist, (size_t)HIST * state_elems(B, c.Nw)));
+    }
     const bool profile = (flags & SNN_PROFILE) != 0;
     r->last_profiled = false;
     r->prof_n = 0;
@@ -1376,6 +1418,8 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
             mark(SNN_REC_KERNEL_ENCODE, false);
         }
         geom.enc_next = fuse_enc && t + 1 < T ? 1 : 0;
+        geom.slot = t % HIST;
+        geom.keep_sh = !geom.fused || t == T - 1 ? 1 : 0;
         mark(SNN_REC_KERNEL_DRIVE, true);
         if (dense)
             k_rec_dense<<<dgrid, GTHREADS, GSMEM, st>>>(r->map_s[0], r->map_s[1], r->map_w, c, d, t, geom,
@@ -1383,6 +1427,10 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
         else
             k_rec_hidden<<<(unsigned)((hid_warps + 7) / 8), 256, 0, st>>>(c, d, t);
         mark(SNN_REC_KERNEL_DRIVE, false);
+        if (dense && (geom.slot == HIST - 1 || t == T - 1)) {
+            const size_t warps = (size_t)((B + 31) / 32) * c.Nw;
+            k_rec_fold<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(c, d, geom.slot + 1);
+        }
         // the tensor form's product adds each step's readout one step later;
         // the run's last step is read out here
         if (!dense || !geom.fused || t == T - 1) {
