@@ -243,6 +243,7 @@ struct TBufs {
     uint16_t* spost;        // [Np][Bp]       excitatory spikes of the step (0/1)
     uint16_t* xpost;        // [NXQ][Np][Bp]  -(nu_pre * x_post), split
     uint32_t* colcnt;       // [N]            excitatory spikes of column j in the step
+    uint32_t* pblk;         // [Np/128][Bp/64] 1 + the last step with a spike in that block of SPOST
     CUtensorMap m_wt, m_sin, m_xpre, m_sint, m_spost, m_xpost;
 };
 

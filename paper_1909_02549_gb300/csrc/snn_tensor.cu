@@ -85,7 +85,8 @@ constexpr uint16_t BF16_ONE = 0x3F80;
 constexpr int TILE_BYTES = 128 * 128;                       // one 128-row x 64-element bfloat16 tile
 constexpr int TC_THREADS = 320;                             // producer, MMA, eight epilogue warps
 constexpr int CUR_STAGES = 3;
-constexpr int DW_STAGES = 2;
+constexpr int DW_SLOTS = 4;
+constexpr int DW_MARKS = 8;                                 // 256 K-blocks: 16384 samples
 constexpr unsigned long long WAIT_NS = 2000000000ull;       // bounded waits: 2 s
 constexpr uint32_t ERR_TENSOR = 4u;                         // device error bit of this form
 
@@ -108,8 +109,10 @@ __device__ __forceinline__ void split_bf16(float x, int n, uint16_t* out) {
 }
 
 __host__ __device__ __forceinline__ int cur_stage_bytes(const TBufs& t) { return t.NW * TILE_BYTES + t.TB * 128; }
-__host__ __device__ __forceinline__ int dw_stage_bytes(const TBufs& t) {
-    return (1 + t.NXQ) * TILE_BYTES + (t.NXP + 1) * t.TNI * 128;
+// a slot of the update's ring: the depression operands, and half of all operands
+__host__ __device__ __forceinline__ int dw_slot_bytes(const TBufs& t) {
+    const int dep = t.NXQ * TILE_BYTES + t.TNI * 128, all = (1 + t.NXQ) * TILE_BYTES + (t.NXP + 1) * t.TNI * 128;
+    return 2 * dep > all ? dep : all / 2;                     // (multiples of 1024: TNI is a multiple of 16)
 }
 
 // ---------------------------------------------------------------- encode ---
@@ -221,7 +224,7 @@ __device__ __forceinline__ void chunk_load(const Consts& c, const Bufs& d, int j
 // of the step.  ncol counts the column's spikes for theta.
 __device__ __forceinline__ void chunk_update(const Consts& c, const Bufs& d, const TBufs& t, int j, int b0,
                                              const float (&I)[16], float th, int p3, int t_local,
-                                             ChunkState& cs, uint32_t& ncol) {
+                                             ChunkState& cs, uint32_t& ncol, uint32_t mark) {
     const int lane = threadIdx.x & 31;
     const bool vj = j < c.N;
     const int nb = c.B - b0 < 16 ? c.B - b0 : 16;            // samples of the chunk (uniform)
@@ -230,40 +233,53 @@ __device__ __forceinline__ void chunk_update(const Consts& c, const Bufs& d, con
     float* xq = cs.xq;
     uint32_t* sw = cs.sw;
     int* C = cs.C;
-    uint32_t fired = 0u;
+    // the sixteen updates, without a branch or a vote between them: their chains
+    // run side by side (a vote per sample had kept them apart)
+    uint32_t fired = 0u, inh = 0u;
 #pragma unroll
     for (int u = 0; u < 16; ++u) {
-        if (u >= nb) break;                                   // uniform over the warp
-        const int b = b0 + u;
-        bool se = false, si = false;
-        if (vj) {
-            const size_t idx = (size_t)b * c.N + j;
-            const uint32_t st = pair_update(c, ve[u], vi[u], sw[u], I[u], C[u], th);
-            se = (st & ST_SE) != 0u;
-            si = (st & ST_SI) != 0u;
-            float x = __fmul_rn(xq[u], c.a_x);
-            x = __fadd_rn(x, se ? 1.0f : 0.0f);
-            xq[u] = x;
+        sw[u] = pair_update(c, ve[u], vi[u], sw[u], I[u], C[u], th);
+        const bool se = (sw[u] & ST_SE) != 0u;
+        xq[u] = __fadd_rn(__fmul_rn(xq[u], c.a_x), se ? 1.0f : 0.0f);
+        fired |= (se ? 1u : 0u) << u;
+        inh |= ((sw[u] & ST_SI) ? 1u : 0u) << u;
+    }
+    const uint32_t live = vj ? (nb < 16 ? (1u << nb) - 1u : 0xFFFFu) : 0u;
+    fired &= live;
+    inh &= live;
+    const size_t i0 = (size_t)b0 * c.N + j;
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+        if ((live >> u) & 1u) {
+            const size_t idx = i0 + (size_t)u * c.N;
             d.v_e[idx] = ve[u];
             d.v_i[idx] = vi[u];
-            d.x_post[idx] = x;
-            d.st[idx] = st;
-            if (se) {
-                d.counts[idx] += 1u;
-                fired |= 1u << u;
-            }
+            d.x_post[idx] = xq[u];
+            d.st[idx] = sw[u];
         }
-        const uint32_t we = __ballot_sync(FULL, se), wi = __ballot_sync(FULL, si);
-        if (lane == 0) {
-            if (wi) atomicAdd(&d.cnt[(size_t)p3 * c.B + b], (uint32_t)__popc(wi));
-            if (c.rec_raster && j < c.N) {                    // lane 0's j starts the warp's 32
-                d.raster_e[((size_t)t_local * c.B + b) * c.Nw + (j >> 5)] = we;
-                d.raster_i[((size_t)t_local * c.B + b) * c.Nw + (j >> 5)] = wi;
-            }
-        }
+    for (uint32_t m = fired; m; m &= m - 1) atomicAdd(&d.counts[i0 + (size_t)(__ffs(m) - 1) * c.N], 1u);   // (one writer)
+    // votes only for the samples in which a neuron of the warp's 32 fired
+    for (uint32_t m = __reduce_or_sync(FULL, inh); m; m &= m - 1) {
+        const int u = __ffs(m) - 1;
+        const uint32_t wi = __ballot_sync(FULL, (inh >> u) & 1u);
+        if (lane == 0) atomicAdd(&d.cnt[(size_t)p3 * c.B + b0 + u], (uint32_t)__popc(wi));
     }
+    if (c.rec_raster)
+        for (int u = 0; u < nb; ++u) {
+            const uint32_t we = __ballot_sync(FULL, (fired >> u) & 1u), wi = __ballot_sync(FULL, (inh >> u) & 1u);
+            if (lane == 0 && j < c.N) {                       // lane 0's j starts the warp's 32
+                const size_t o = ((size_t)t_local * c.B + b0 + u) * c.Nw + (j >> 5);
+                d.raster_e[o] = we;
+                d.raster_i[o] = wi;
+            }
+        }
     if (!vj) return;
-    if (fired) atomicOr(&d.spkT[(size_t)j * c.Bw + (b0 >> 5)], fired << (b0 & 31));
+    if (fired) {
+        atomicOr(&d.spkT[(size_t)j * c.Bw + (b0 >> 5)], fired << (b0 & 31));
+        // this block of SPOST is not zero in this step (a stale mark of the same
+        // step only costs the update a product with zeros)
+        t.pblk[(size_t)(j >> 7) * (t.Bp / KB) + b0 / KB] = mark;
+    }
     ncol += (uint32_t)__popc(fired);
     if (!c.learn) return;
     // the update's operands: spikes and -(nu_pre * x_post) of the 16 samples
@@ -404,7 +420,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_current(const __grid_consta
 #pragma unroll
                 for (int u = 0; u < 16; ++u) I[u] = __uint_as_float(r[u]);
                 if (ch != half) chunk_load(c, d, j, b0, p3, cs);   // the first chunk is in flight already
-                chunk_update(c, d, t, j, b0, I, th, p3, t_local, cs, ncol);
+                chunk_update(c, d, t, j, b0, I, th, p3, t_local, cs, ncol, (uint32_t)tt + 1u);
             }
             if (c.learn && ncol && j < c.N) atomicAdd(&t.colcnt[j], ncol);
         }
@@ -450,7 +466,7 @@ __global__ void __launch_bounds__(128) k_t_gcurrent(Consts c, Bufs d, TBufs t, i
             }
             I[u] = acc;
         }
-        chunk_update(c, d, t, j, b0, I, th, p3, t_local, cs, ncol);
+        chunk_update(c, d, t, j, b0, I, th, p3, t_local, cs, ncol, (uint32_t)tt + 1u);
     }
     if (c.learn && ncol && j < c.N) atomicAdd(&t.colcnt[j], ncol);
 }
@@ -496,10 +512,20 @@ __device__ __forceinline__ void wchunk_update(const Consts& c, const Bufs& d, co
                                               const float (&D)[16], WChunk<MASTER>& wc) {
     if (j >= c.N) return;
     const int nu = c.n_in - i0 < 16 ? c.n_in - i0 : 16;
+    float dm[16];                                             // the reduced update; one choice for all sixteen
+    if (c.reduce != SNN_REDUCE_MEAN) {
+#pragma unroll
+        for (int u = 0; u < 16; ++u) dm[u] = D[u];
+    } else if (c.B_pow2) {
+#pragma unroll
+        for (int u = 0; u < 16; ++u) dm[u] = __fmul_rn(D[u], c.inv_B);
+    } else {
+#pragma unroll
+        for (int u = 0; u < 16; ++u) dm[u] = __fdiv_rn(D[u], (float)c.B);
+    }
 #pragma unroll
     for (int u = 0; u < 16; ++u) {
-        float x = D[u];
-        if (c.reduce == SNN_REDUCE_MEAN) x = batch_mean(c, x);
+        const float x = dm[u];
         const size_t k = (size_t)(i0 + u) * c.N + j;
         float w = wc.w[u];
         if (MASTER) {
@@ -529,18 +555,45 @@ __device__ __forceinline__ void wchunk_update(const Consts& c, const Bufs& d, co
     }
 }
 
+// The ring of k_t_dw: DW_SLOTS slots, each the depression operands of a K-block
+// (XPOST, SINT); a block whose neurons fired also takes the slot after an even
+// one for the potentiation operands (SPOST, XPRE).  Without a post spike the
+// potentiation product is exactly zero, so neither loaded nor computed: three of
+// the five products and more than half of the bytes of 73 % of the blocks at
+// 784->6400 (most steps only a few of the neurons fire).  next: the slot of the
+// next block; uses, fills: how often a slot was taken, and filled by its own block
+// (its barriers' phases).
+struct SlotWalk {
+    int pos = 0;
+    uint32_t n = 0u, f = 0u;              // a byte per slot (phases need the low bit)
+    __device__ __forceinline__ int next(bool post) const { return post ? (pos + 1) & ~1 & (DW_SLOTS - 1) : pos; }
+    __device__ __forceinline__ uint32_t uses(int s) const { return (n >> (8 * s)) & 0xFFu; }
+    __device__ __forceinline__ uint32_t fills(int s) const { return (f >> (8 * s)) & 0xFFu; }
+    __device__ __forceinline__ void take(int s, bool post) {
+        bump(n, s);
+        bump(f, s);
+        if (post) bump(n, s + 1);
+        pos = (s + (post ? 2 : 1)) & (DW_SLOTS - 1);
+    }
+    // counts 1, 2, 3, 2, 3 ...: the low bit alternates and never returns to 0 uses
+    __device__ __forceinline__ void bump(uint32_t& v, int s) {
+        const uint32_t x = (v >> (8 * s)) & 0xFFu;
+        v = (v & ~(0xFFu << (8 * s))) | ((x < 3u ? x + 1u : 2u) << (8 * s));
+    }
+};
+
 template <bool MASTER>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ CUtensorMap mSP,
                                                         const __grid_constant__ CUtensorMap mXQ,
                                                         const __grid_constant__ CUtensorMap mXP,
                                                         const __grid_constant__ CUtensorMap mSIT,
-                                                        Consts c, Bufs d, TBufs t) {
+                                                        Consts c, Bufs d, TBufs t, int t_local) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const int SB = dw_stage_bytes(t);
-    uint64_t* full = (uint64_t*)(smem + DW_STAGES * SB);
-    uint64_t* empty = full + DW_STAGES;
-    uint64_t* accf = empty + DW_STAGES;
+    const int SLOT = dw_slot_bytes(t);
+    uint64_t* full = (uint64_t*)(smem + DW_SLOTS * SLOT);
+    uint64_t* empty = full + DW_SLOTS;
+    uint64_t* accf = empty + DW_SLOTS;
     uint64_t* drain = accf + 1;
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -549,19 +602,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
     const int nkb = t.Bp / KB;
     const int k0 = (int)((long long)ks * nkb / t.KS), k1 = (int)((long long)(ks + 1) * nkb / t.KS);
     const int nk = k1 - k0;
-    const int BT = (1 + t.NXQ) * TILE_BYTES, BTI = t.TNI * 128;   // offset of the B tiles, B tile bytes
+    const int BTI = t.TNI * 128;                                  // bytes of a B tile
     const int PS = t.TNI + 4;                                     // row stride of the partial tile
     if (tid == 0) {
-        for (int s = 0; s < DW_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        for (int s = 0; s < DW_SLOTS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         mbar_init(accf, 1);
         mbar_init(drain, 1);
         mbar_fence_init();
     }
+    // which of the slice's K-blocks have a post spike in this neuron tile: bit k
+    // of the first 32 * DW_MARKS (the rest count as having one)
+    __shared__ uint32_t s_post[DW_MARKS];
+    if (tid < DW_MARKS) s_post[tid] = 0u;
+    __syncthreads();
+    const uint32_t mark = (uint32_t)(d.step[0] + (unsigned long long)t_local) + 1u;
+    for (int k = tid; k < nk && k < 32 * DW_MARKS; k += TC_THREADS)
+        if (t.pblk[(size_t)tm * nkb + k0 + k] == mark) atomicOr(&s_post[k >> 5], 1u << (k & 31));
     if (warp == 1) tmem_alloc(&s_tmem, ncols);
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = s_tmem;
+    auto has_post = [&](int k) { return k >= 32 * DW_MARKS || ((s_post[k >> 5] >> (k & 31)) & 1u) != 0u; };
     // the epilogue thread's neuron and 16-input chunks: ks + KS * (half + 2m)
     const int quarter = warp & 3, half = (warp - 2) >> 2;
     const int row = quarter * 32 + lane;
@@ -571,42 +633,68 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
     WChunk<MASTER> wc;
     if (warp == 0) {
         if (lane == 0) {                                      // TMA producer
-            int it = 0;
+            SlotWalk sw;
             bool ok = true;
-            for (; it < nk; ++it) {
-                if (!(ok = stage_free(empty, it, DW_STAGES))) break;
-                uint8_t* st = smem + (it % DW_STAGES) * SB;
-                uint64_t* f = &full[it % DW_STAGES];
+            uint32_t used = 0u;                               // slots ever filled
+            for (int it = 0; it < nk; ++it) {
+                const bool post = has_post(it);
+                const int s = sw.next(post);
+                // (a block with post spikes takes two slots; both were freed with
+                // the block that held them)
+                if (sw.uses(s) > 0) ok = mbar_wait(&empty[s], (sw.uses(s) - 1) & 1, WAIT_NS);
+                if (ok && post && sw.uses(s + 1) > 0) ok = mbar_wait(&empty[s + 1], (sw.uses(s + 1) - 1) & 1, WAIT_NS);
+                if (!ok) break;
+                uint8_t* st = smem + s * SLOT;
+                uint64_t* f = &full[s];
                 const int kx = (k0 + it) * KB;
-                mbar_expect_tx(f, (uint32_t)SB);
-                tma_2d(st, &mSP, kx, tm * 128, f);
-                for (int q = 0; q < t.NXQ; ++q) tma_2d(st + (1 + q) * TILE_BYTES, &mXQ, kx, q * t.Np + tm * 128, f);
-                for (int p = 0; p < t.NXP; ++p) tma_2d(st + BT + p * BTI, &mXP, kx, p * c.n_in + tn * t.TNI, f);
-                tma_2d(st + BT + t.NXP * BTI, &mSIT, kx, tn * t.TNI, f);
+                mbar_expect_tx(f, (uint32_t)(t.NXQ * TILE_BYTES + BTI + (post ? TILE_BYTES + t.NXP * BTI : 0)));
+                for (int q = 0; q < t.NXQ; ++q) tma_2d(st + q * TILE_BYTES, &mXQ, kx, q * t.Np + tm * 128, f);
+                st += t.NXQ * TILE_BYTES;
+                tma_2d(st, &mSIT, kx, tn * t.TNI, f);
+                st += BTI;
+                if (post) {
+                    tma_2d(st, &mSP, kx, tm * 128, f);
+                    st += TILE_BYTES;
+                    for (int p = 0; p < t.NXP; ++p) tma_2d(st + p * BTI, &mXP, kx, p * c.n_in + tn * t.TNI, f);
+                }
+                used |= 1u << s;
+                sw.take(s, post);
             }
             if (!ok) atomicOr(d.err, ERR_TENSOR);
-            drain_loads(full, it, DW_STAGES);
+            // every copy issued has landed before the CTA may leave
+            for (int s = 0; s < DW_SLOTS; ++s)
+                if ((used >> s) & 1u) mbar_wait(&full[s], (sw.fills(s) - 1) & 1, WAIT_NS);
         }
     } else if (warp == 1) {
         if (lane == 0) {                                      // MMA issuer
             const uint32_t idesc = idesc_bf16(t.TNI);
+            SlotWalk sw;
             bool ok = true;
             for (int it = 0; it < nk; ++it) {
-                const int s = it % DW_STAGES;
-                if (!(ok = mbar_wait(&full[s], (it / DW_STAGES) & 1, WAIT_NS))) break;
+                const bool post = has_post(it);
+                const int s = sw.next(post);
+                if (!(ok = mbar_wait(&full[s], sw.fills(s) & 1, WAIT_NS))) break;
                 fence_after();
-                const uint32_t a0 = su32(smem + s * SB), b0 = a0 + BT;
-                const uint32_t sit = b0 + t.NXP * BTI;
+                const uint32_t xq = su32(smem + s * SLOT), sit = xq + t.NXQ * TILE_BYTES;
+                const uint32_t sp = sit + BTI, xp = sp + TILE_BYTES;
 #pragma unroll
                 for (int k = 0; k < KB / 16; ++k) {
-                    for (int p = 0; p < t.NXP; ++p)           // potentiation: SPOST . XPRE_p
-                        mma_bf16(tmem, sdesc(a0) + (uint64_t)(2 * k), sdesc(b0 + p * BTI) + (uint64_t)(2 * k),
-                                 idesc, (it | k | p) != 0 ? 1u : 0u);
-                    for (int q = 0; q < t.NXQ; ++q)           // depression: XPOST_q . SINT
-                        mma_bf16(tmem, sdesc(a0 + (1 + q) * TILE_BYTES) + (uint64_t)(2 * k), sdesc(sit) + (uint64_t)(2 * k),
-                                 idesc, 1u);
+                    uint32_t acc = it | k;
+                    if (post)
+                        for (int p = 0; p < t.NXP; ++p) {     // potentiation: SPOST . XPRE_p
+                            mma_bf16(tmem, sdesc(sp) + (uint64_t)(2 * k), sdesc(xp + p * BTI) + (uint64_t)(2 * k),
+                                     idesc, acc != 0 ? 1u : 0u);
+                            acc = 1u;
+                        }
+                    for (int q = 0; q < t.NXQ; ++q) {         // depression: XPOST_q . SINT
+                        mma_bf16(tmem, sdesc(xq + q * TILE_BYTES) + (uint64_t)(2 * k), sdesc(sit) + (uint64_t)(2 * k),
+                                 idesc, acc != 0 ? 1u : 0u);
+                        acc = 1u;
+                    }
                 }
                 mma_commit(&empty[s]);
+                if (post) mma_commit(&empty[s + 1]);
+                sw.take(s, post);
             }
             if (ok) mma_commit(accf);
             else atomicOr(d.err, ERR_TENSOR);
@@ -780,6 +868,7 @@ size_t tensor_bytes(const TBufs& t, const Consts& c) {
     n += up((size_t)t.Np * t.Bp * 2, 256);
     n += up((size_t)t.NXQ * t.Np * t.Bp * 2, 256);
     n += up((size_t)c.N * 4, 256);
+    n += up((size_t)(t.Np / 128) * (t.Bp / KB) * 4, 256);
     return n;
 }
 
@@ -793,6 +882,7 @@ bool tensor_bind(TBufs& t, const Consts& c, void* base) {
     t.spost = (uint16_t*)take((size_t)t.Np * t.Bp * 2);
     t.xpost = (uint16_t*)take((size_t)t.NXQ * t.Np * t.Bp * 2);
     t.colcnt = (uint32_t*)take((size_t)c.N * 4);
+    t.pblk = (uint32_t*)take((size_t)(t.Np / 128) * (t.Bp / KB) * 4);
     return encode_bf16_map(&t.m_wt, t.wt, t.NW * t.Np, t.Kp, 128) &&
            encode_bf16_map(&t.m_sin, t.sin, t.Bp, t.Kp, t.TB) &&
            encode_bf16_map(&t.m_xpre, t.xpre, t.NXP * c.n_in, t.Bp, t.TNI) &&
@@ -812,7 +902,7 @@ cudaError_t launch_tensor_begin(const Consts& c, const Bufs& d, const TBufs& t, 
 // terms and 128 samples; three A tiles and four B tiles of 128 inputs): set
 // once per device, under a lock shared by every host thread.
 constexpr int CUR_SMEM_MAX = CUR_STAGES * (3 * TILE_BYTES + 128 * 128) + 1024 + 64;
-constexpr int DW_SMEM_MAX = DW_STAGES * (4 * TILE_BYTES + 3 * 128 * 128) + 1024 + 64;
+constexpr int DW_SMEM_MAX = DW_SLOTS * (4 * TILE_BYTES + 3 * 128 * 128) / 2 + 1024 + 128;
 static_assert(DW_SMEM_MAX <= 232448 && CUR_SMEM_MAX <= 232448, "227 KB of shared memory per CTA");
 
 cudaError_t ensure_attributes() {
@@ -854,7 +944,7 @@ cudaError_t launch_tensor_step(const Consts& c, const Bufs& d, const TBufs& t, i
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(t.Np / 128, t.nti, t.KS);
         cfg.blockDim = dim3(TC_THREADS);
-        cfg.dynamicSmemBytes = (size_t)DW_STAGES * dw_stage_bytes(t) + 1024 + 64;
+        cfg.dynamicSmemBytes = (size_t)DW_SLOTS * dw_slot_bytes(t) + 1024 + 128;
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -863,8 +953,8 @@ cudaError_t launch_tensor_step(const Consts& c, const Bufs& d, const TBufs& t, i
         at[0].val.clusterDim.z = (unsigned)t.KS;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        if (c.wmaster) TT_TRY(cudaLaunchKernelEx(&cfg, k_t_dw<true>, t.m_spost, t.m_xpost, t.m_xpre, t.m_sint, c, d, t));
-        else TT_TRY(cudaLaunchKernelEx(&cfg, k_t_dw<false>, t.m_spost, t.m_xpost, t.m_xpre, t.m_sint, c, d, t));
+        if (c.wmaster) TT_TRY(cudaLaunchKernelEx(&cfg, k_t_dw<true>, t.m_spost, t.m_xpost, t.m_xpre, t.m_sint, c, d, t, t_local));
+        else TT_TRY(cudaLaunchKernelEx(&cfg, k_t_dw<false>, t.m_spost, t.m_xpost, t.m_xpre, t.m_sint, c, d, t, t_local));
         TT_TRY(prof_stop(prof, s));
     }
     return cudaSuccess;
