@@ -235,6 +235,7 @@ struct TBufs {
     int Np, Kp, Bp;         // neurons padded to 128, inputs to 64, samples to 64
     int TB;                 // samples per tile of the current
     int TNI, nti, KS;       // update: inputs per tile, input tiles, batch slices
+    int sms;                // multiprocessors: the products' persistent grids
     int dense;              // 1: the current is the tcgen05 product; 0: the ordered gather
     uint16_t* wt;           // [NW][Np][Kp]   W transposed, split
     uint16_t* sin;          // [Bp][Kp]       input spikes of the step (0/1)

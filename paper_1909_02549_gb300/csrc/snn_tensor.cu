@@ -83,7 +83,8 @@ using namespace tc;
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr uint16_t BF16_ONE = 0x3F80;
 constexpr int TILE_BYTES = 128 * 128;                       // one 128-row x 64-element bfloat16 tile
-constexpr int TC_THREADS = 320;                             // producer, MMA, eight epilogue warps
+constexpr int EPI_WARPS = 8;
+constexpr int TC_THREADS = 64 + 32 * EPI_WARPS;             // producer, MMA, epilogue warps
 constexpr int CUR_STAGES = 3;
 constexpr int DW_SLOTS = 4;
 constexpr int DW_MARKS = 8;                                 // 256 K-blocks: 16384 samples
@@ -319,6 +320,9 @@ __device__ __forceinline__ float threshold_of(const Consts& c, const Bufs& d, in
 
 // ------------------------------------------------------------- the current ---
 
+// Tensor-memory columns of an accumulator of n columns.
+__device__ __forceinline__ uint32_t acc_cols(int n) { return n <= 32 ? 32u : n <= 64 ? 64u : n <= 128 ? 128u : 256u; }
+
 // Producer side of a pipeline: waits until stage s may be refilled (bounded).
 __device__ __forceinline__ bool stage_free(uint64_t* empty, int it, int S) {
     if (it < S) return true;
@@ -332,7 +336,15 @@ __device__ __forceinline__ void drain_loads(uint64_t* full, int issued, int S) {
         mbar_wait(&full[it % S], (it / S) & 1, WAIT_NS);
 }
 
-// grid (Np/128 neuron tiles, ceil(B/TB) sample tiles), TC_THREADS threads.
+// Persistent: a CTA per SM walks the tiles of 128 neurons x TB samples (tile =
+// blockIdx.x + i * gridDim.x, neuron tiles fastest) with two accumulators in tensor
+// memory, so that a tile's product runs during the epilogue of the tile before.
+// What bounds it: the epilogue (state read and written, 32 bytes a neuron and
+// sample, and the updates' instructions; 11 to 22 us a tile of 128 samples) and
+// the operands' way from L2.  784->6400, B = 1024, a step of 250: with a launch of
+// 400 CTAs, product (8 to 14 us) and epilogue one after the other, 55.3 ms a run;
+// 49.0 with the epilogue's chains side by side; 44.5 with this overlap here and in
+// k_t_dw (BF16 at B = 256: 21.1, 19.7 and 16.4 ms).
 __global__ void __launch_bounds__(TC_THREADS, 1) k_t_current(const __grid_constant__ CUtensorMap mW,
                                                              const __grid_constant__ CUtensorMap mS,
                                                              Consts c, Bufs d, TBufs t, int t_local) {
@@ -341,37 +353,41 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_current(const __grid_consta
     const int SB = cur_stage_bytes(t);
     uint64_t* full = (uint64_t*)(smem + CUR_STAGES * SB);
     uint64_t* empty = full + CUR_STAGES;
-    uint64_t* accf = empty + CUR_STAGES;
-    uint64_t* drain = accf + 1;
+    uint64_t* accf = empty + CUR_STAGES;                      // [2] accumulator ready
+    uint64_t* acce = accf + 2;                                // [2] accumulator drained
+    uint64_t* drain = acce + 2;
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tm = blockIdx.x, tbi = blockIdx.y;
-    const uint32_t ncols = t.TB <= 32 ? 32u : t.TB <= 64 ? 64u : t.TB <= 128 ? 128u : 256u;
+    const uint32_t ncols = acc_cols(t.TB);
     if (tid == 0) {
         for (int s = 0; s < CUR_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        mbar_init(accf, 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(&accf[i], 1); mbar_init(&acce[i], EPI_WARPS); }
         mbar_init(drain, 1);
         mbar_fence_init();
     }
-    if (warp == 1) tmem_alloc(&s_tmem, ncols);
+    if (warp == 1) tmem_alloc(&s_tmem, 2 * ncols);
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = s_tmem;
     const int nk = t.Kp / KB;
+    const int ntm = t.Np / 128, ntiles = ntm * ((c.B + t.TB - 1) / t.TB);
     const unsigned long long tt = d.step[0] + (unsigned long long)t_local;
     const int p3 = (int)(tt % 3ull);
     if (warp == 0) {
         if (lane == 0) {                                      // TMA producer
             int it = 0;
             bool ok = true;
-            for (; it < nk; ++it) {
-                if (!(ok = stage_free(empty, it, CUR_STAGES))) break;
-                uint8_t* st = smem + (it % CUR_STAGES) * SB;
-                uint64_t* f = &full[it % CUR_STAGES];
-                mbar_expect_tx(f, (uint32_t)SB);
-                for (int w = 0; w < t.NW; ++w) tma_2d(st + w * TILE_BYTES, &mW, it * KB, w * t.Np + tm * 128, f);
-                tma_2d(st + t.NW * TILE_BYTES, &mS, it * KB, tbi * t.TB, f);
+            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+                const int tm = tile % ntm, tbi = tile / ntm;
+                for (int kb = 0; kb < nk; ++kb, ++it) {
+                    if (!(ok = stage_free(empty, it, CUR_STAGES))) break;
+                    uint8_t* st = smem + (it % CUR_STAGES) * SB;
+                    uint64_t* f = &full[it % CUR_STAGES];
+                    mbar_expect_tx(f, (uint32_t)SB);
+                    for (int w = 0; w < t.NW; ++w) tma_2d(st + w * TILE_BYTES, &mW, kb * KB, w * t.Np + tm * 128, f);
+                    tma_2d(st + t.NW * TILE_BYTES, &mS, kb * KB, tbi * t.TB, f);
+                }
             }
             if (!ok) atomicOr(d.err, ERR_TENSOR);
             drain_loads(full, it, CUR_STAGES);
@@ -379,37 +395,48 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_current(const __grid_consta
     } else if (warp == 1) {
         if (lane == 0) {                                      // MMA issuer
             const uint32_t idesc = idesc_bf16(t.TB);
+            int it = 0, lt = 0;
             bool ok = true;
-            for (int it = 0; it < nk; ++it) {
-                const int s = it % CUR_STAGES;
-                if (!(ok = mbar_wait(&full[s], (it / CUR_STAGES) & 1, WAIT_NS))) break;
+            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++lt) {
+                const int buf = lt & 1;
+                if (lt >= 2 && !(ok = mbar_wait(&acce[buf], ((lt >> 1) - 1) & 1, WAIT_NS))) break;
                 fence_after();
-                const uint32_t a0 = su32(smem + s * SB), b0 = a0 + t.NW * TILE_BYTES;
+                const uint32_t acc = tmem + (uint32_t)buf * ncols;
+                for (int kb = 0; kb < nk; ++kb, ++it) {
+                    const int s = it % CUR_STAGES;
+                    if (!(ok = mbar_wait(&full[s], (it / CUR_STAGES) & 1, WAIT_NS))) break;
+                    fence_after();
+                    const uint32_t a0 = su32(smem + s * SB), b0 = a0 + t.NW * TILE_BYTES;
 #pragma unroll
-                for (int k = 0; k < KB / 16; ++k)
-                    for (int w = 0; w < t.NW; ++w)
-                        mma_bf16(tmem, sdesc(a0 + w * TILE_BYTES) + (uint64_t)(2 * k), sdesc(b0) + (uint64_t)(2 * k),
-                                 idesc, (it | k | w) != 0 ? 1u : 0u);
-                mma_commit(&empty[s]);
+                    for (int k = 0; k < KB / 16; ++k)
+                        for (int w = 0; w < t.NW; ++w)
+                            mma_bf16(acc, sdesc(a0 + w * TILE_BYTES) + (uint64_t)(2 * k), sdesc(b0) + (uint64_t)(2 * k),
+                                     idesc, (kb | k | w) != 0 ? 1u : 0u);
+                    mma_commit(&empty[s]);
+                }
+                if (ok) mma_commit(&accf[buf]);
             }
-            if (ok) mma_commit(accf);
-            else atomicOr(d.err, ERR_TENSOR);
+            if (!ok) atomicOr(d.err, ERR_TENSOR);
             mma_commit(drain);                                // every MMA issued has completed
             if (!mbar_wait(drain, 0, WAIT_NS)) atomicOr(d.err, ERR_TENSOR);
         }
     } else {                                                  // epilogue: neuron update
         const int quarter = warp & 3, half = (warp - 2) >> 2;
-        const int j = tm * 128 + quarter * 32 + lane;
-        ChunkState cs;
-        const int bfirst = tbi * t.TB + half * 16;
-        if (bfirst < c.B) chunk_load(c, d, j, bfirst, p3, cs);   // overlaps the product
-        const bool got = __all_sync(FULL, mbar_wait(accf, 0, WAIT_NS) ? 1 : 0) != 0;
-        if (!got) {
-            if (lane == 0) atomicOr(d.err, ERR_TENSOR);
-        } else {
+        int lt = 0;
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++lt) {
+            const int tm = tile % ntm, tbi = tile / ntm, buf = lt & 1;
+            const int j = tm * 128 + quarter * 32 + lane;
+            ChunkState cs;
+            const int bfirst = tbi * t.TB + half * 16;
+            if (bfirst < c.B) chunk_load(c, d, j, bfirst, p3, cs);   // overlaps the product
+            const bool got = __all_sync(FULL, mbar_wait(&accf[buf], (lt >> 1) & 1, WAIT_NS) ? 1 : 0) != 0;
+            if (!got) {
+                if (lane == 0) atomicOr(d.err, ERR_TENSOR);
+                break;
+            }
             fence_after();
             const float th = threshold_of(c, d, j);
-            const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16);
+            const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * ncols;
             uint32_t ncol = 0u;
             for (int ch = half; ch < t.TB / 16; ch += 2) {
                 const int b0 = tbi * t.TB + ch * 16;
@@ -422,6 +449,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_current(const __grid_consta
                 if (ch != half) chunk_load(c, d, j, b0, p3, cs);   // the first chunk is in flight already
                 chunk_update(c, d, t, j, b0, I, th, p3, t_local, cs, ncol, (uint32_t)tt + 1u);
             }
+            fence_before();                                   // this warp is done with the accumulator
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acce[buf]);
             if (c.learn && ncol && j < c.N) atomicAdd(&t.colcnt[j], ncol);
         }
     }
@@ -429,7 +459,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_current(const __grid_consta
     __syncthreads();
     if (warp == 1) {
         fence_after();
-        tmem_free(tmem, ncols);
+        tmem_free(tmem, 2 * ncols);
     }
 }
 
@@ -473,10 +503,12 @@ __global__ void __launch_bounds__(128) k_t_gcurrent(Consts c, Bufs d, TBufs t, i
 
 // --------------------------------------------------------------- the update ---
 
-// grid (Np/128 neuron tiles, nti input tiles of TNI, KS batch slices),
-// clusters of the KS slices of one tile, TC_THREADS threads.  Each CTA
-// accumulates its slice of the batch in tensor memory.  With one slice its
-// epilogue applies the update straight from the accumulator; otherwise every
+// Tiles of 128 neurons x TNI inputs, KS batch slices, TC_THREADS threads.  Each
+// CTA accumulates its slice of the batch in tensor memory.  With one slice a CTA
+// per SM walks the tiles with two accumulators, its epilogue applying a tile's
+// update straight from the accumulator while the next tile's product runs;
+// otherwise the grid is (neuron tiles, input tiles, slices) in clusters of the
+// slices of a tile, and every
 // CTA leaves its partial tile in shared memory, and after a cluster barrier CTA
 // k updates the 16-input chunks k, k+KS, ... of the tile, adding the slices'
 // partial tiles in slice order through distributed shared memory (a second
@@ -560,29 +592,28 @@ __device__ __forceinline__ void wchunk_update(const Consts& c, const Bufs& d, co
 // one for the potentiation operands (SPOST, XPRE).  Without a post spike the
 // potentiation product is exactly zero, so neither loaded nor computed: three of
 // the five products and more than half of the bytes of 73 % of the blocks at
-// 784->6400 (most steps only a few of the neurons fire).  next: the slot of the
-// next block; uses, fills: how often a slot was taken, and filled by its own block
-// (its barriers' phases).
+// 784->6400 (most steps only a few of the neurons fire).
 struct SlotWalk {
     int pos = 0;
-    uint32_t n = 0u, f = 0u;              // a byte per slot (phases need the low bit)
+    uint32_t taken = 0u, np = 0u, fp = 0u;   // slots ever taken; parities of a slot's uses, and of its fills
     __device__ __forceinline__ int next(bool post) const { return post ? (pos + 1) & ~1 & (DW_SLOTS - 1) : pos; }
-    __device__ __forceinline__ uint32_t uses(int s) const { return (n >> (8 * s)) & 0xFFu; }
-    __device__ __forceinline__ uint32_t fills(int s) const { return (f >> (8 * s)) & 0xFFu; }
+    __device__ __forceinline__ bool was_taken(int s) const { return ((taken >> s) & 1u) != 0u; }
+    __device__ __forceinline__ uint32_t last_use(int s) const { return ((np >> s) & 1u) ^ 1u; }    // its phase's parity
+    __device__ __forceinline__ uint32_t next_fill(int s) const { return (fp >> s) & 1u; }
+    __device__ __forceinline__ uint32_t last_fill(int s) const { return next_fill(s) ^ 1u; }
     __device__ __forceinline__ void take(int s, bool post) {
-        bump(n, s);
-        bump(f, s);
-        if (post) bump(n, s + 1);
+        const uint32_t m = (post ? 3u : 1u) << s;
+        taken |= m;
+        np ^= m;
+        fp ^= 1u << s;
         pos = (s + (post ? 2 : 1)) & (DW_SLOTS - 1);
-    }
-    // counts 1, 2, 3, 2, 3 ...: the low bit alternates and never returns to 0 uses
-    __device__ __forceinline__ void bump(uint32_t& v, int s) {
-        const uint32_t x = (v >> (8 * s)) & 0xFFu;
-        v = (v & ~(0xFFu << (8 * s))) | ((x < 3u ? x + 1u : 2u) << (8 * s));
     }
 };
 
-template <bool MASTER>
+// SLICED: KS > 1 (instantiations of their own: the kernels alternate within a step,
+// and each launch fetches its code anew; one for both cost narrow layers 0.7 us a
+// step).
+template <bool MASTER, bool SLICED>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ CUtensorMap mSP,
                                                         const __grid_constant__ CUtensorMap mXQ,
                                                         const __grid_constant__ CUtensorMap mXP,
@@ -593,56 +624,75 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
     const int SLOT = dw_slot_bytes(t);
     uint64_t* full = (uint64_t*)(smem + DW_SLOTS * SLOT);
     uint64_t* empty = full + DW_SLOTS;
-    uint64_t* accf = empty + DW_SLOTS;
-    uint64_t* drain = accf + 1;
+    uint64_t* accf = empty + DW_SLOTS;                            // [2] accumulator ready
+    uint64_t* acce = accf + 2;                                    // [2] accumulator drained
+    uint64_t* drain = acce + 2;
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tm = blockIdx.x, tn = blockIdx.y, ks = blockIdx.z;
-    const uint32_t ncols = t.TNI <= 32 ? 32u : t.TNI <= 64 ? 64u : t.TNI <= 128 ? 128u : 256u;
+    const int ks = blockIdx.z;
+    const uint32_t ncols = acc_cols(t.TNI);
     const int nkb = t.Bp / KB;
     const int k0 = (int)((long long)ks * nkb / t.KS), k1 = (int)((long long)(ks + 1) * nkb / t.KS);
     const int nk = k1 - k0;
     const int BTI = t.TNI * 128;                                  // bytes of a B tile
     const int PS = t.TNI + 4;                                     // row stride of the partial tile
+    // tiles, neuron tiles fastest: with one slice the CTA's are first, first + step,
+    // ...; with more, its cluster's one
+    const int ntm = t.Np / 128, ntiles = ntm * t.nti;
+    auto tile_m = [&](int tile) { return SLICED ? (int)blockIdx.x : tile % ntm; };
+    auto tile_n = [&](int tile) { return SLICED ? (int)blockIdx.y : tile / ntm; };
+    const int first = SLICED ? 0 : (int)blockIdx.x, end = SLICED ? 1 : ntiles, step = SLICED ? 1 : (int)gridDim.x;
     if (tid == 0) {
         for (int s = 0; s < DW_SLOTS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        mbar_init(accf, 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(&accf[i], 1); mbar_init(&acce[i], EPI_WARPS); }
         mbar_init(drain, 1);
         mbar_fence_init();
     }
-    // which of the slice's K-blocks have a post spike in this neuron tile: bit k
-    // of the first 32 * DW_MARKS (the rest count as having one)
-    __shared__ uint32_t s_post[DW_MARKS];
-    if (tid < DW_MARKS) s_post[tid] = 0u;
-    __syncthreads();
-    const uint32_t mark = (uint32_t)(d.step[0] + (unsigned long long)t_local) + 1u;
-    for (int k = tid; k < nk && k < 32 * DW_MARKS; k += TC_THREADS)
-        if (t.pblk[(size_t)tm * nkb + k0 + k] == mark) atomicOr(&s_post[k >> 5], 1u << (k & 31));
-    if (warp == 1) tmem_alloc(&s_tmem, ncols);
+    if (warp == 1) tmem_alloc(&s_tmem, 2 * ncols);
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = s_tmem;
-    auto has_post = [&](int k) { return k >= 32 * DW_MARKS || ((s_post[k >> 5] >> (k & 31)) & 1u) != 0u; };
+    // which of the slice's K-blocks have a post spike in neuron tile tm: bit k of
+    // the first 32 * DW_MARKS (the rest count as having one); a copy each for the
+    // producer's and the MMA warp.  With several slices the layer is narrow: most
+    // blocks have one, and a CTA's few would wait for the marks' load (784->626,
+    // B = 626: 1.3 % over a run), so all count as having one.
+    constexpr bool marked = !SLICED;
+    __shared__ uint32_t s_post[2][DW_MARKS];
+    auto read_marks = [&](int tm) {                               // (whole warp)
+        if (!marked) return;
+        const uint32_t mark = (uint32_t)(d.step[0] + (unsigned long long)t_local) + 1u;
+        __syncwarp();
+        for (int k = 0; k < nk && k < 32 * DW_MARKS; k += 32) {
+            const bool p = k + lane < nk && t.pblk[(size_t)tm * nkb + k0 + k + lane] == mark;
+            const uint32_t m = __ballot_sync(FULL, p);
+            if (lane == 0) s_post[warp][k >> 5] = m;
+        }
+        __syncwarp();
+    };
+    auto has_post = [&](int k) { return !marked || k >= 32 * DW_MARKS || ((s_post[warp][k >> 5] >> (k & 31)) & 1u) != 0u; };
     // the epilogue thread's neuron and 16-input chunks: ks + KS * (half + 2m)
     const int quarter = warp & 3, half = (warp - 2) >> 2;
     const int row = quarter * 32 + lane;
-    const int j = tm * 128 + row;
     const int nch = t.TNI / 16;
     const int ch0 = ks + t.KS * half, chs = 2 * t.KS;
     WChunk<MASTER> wc;
-    if (warp == 0) {
-        if (lane == 0) {                                      // TMA producer
-            SlotWalk sw;
-            bool ok = true;
-            uint32_t used = 0u;                               // slots ever filled
-            for (int it = 0; it < nk; ++it) {
+    if (warp == 0) {                                          // TMA producer (lane 0)
+        SlotWalk sw;
+        bool ok = true;
+        uint32_t used = 0u;                                   // slots ever filled
+        for (int tile = first; tile < end; tile += step) {
+            const int tm = tile_m(tile), tn = tile_n(tile);
+            read_marks(tm);
+            if (lane != 0) continue;
+            for (int it = 0; it < nk && ok; ++it) {
                 const bool post = has_post(it);
                 const int s = sw.next(post);
                 // (a block with post spikes takes two slots; both were freed with
                 // the block that held them)
-                if (sw.uses(s) > 0) ok = mbar_wait(&empty[s], (sw.uses(s) - 1) & 1, WAIT_NS);
-                if (ok && post && sw.uses(s + 1) > 0) ok = mbar_wait(&empty[s + 1], (sw.uses(s + 1) - 1) & 1, WAIT_NS);
+                if (sw.was_taken(s)) ok = mbar_wait(&empty[s], sw.last_use(s), WAIT_NS);
+                if (ok && post && sw.was_taken(s + 1)) ok = mbar_wait(&empty[s + 1], sw.last_use(s + 1), WAIT_NS);
                 if (!ok) break;
                 uint8_t* st = smem + s * SLOT;
                 uint64_t* f = &full[s];
@@ -660,20 +710,29 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
                 used |= 1u << s;
                 sw.take(s, post);
             }
+        }
+        if (lane == 0) {
             if (!ok) atomicOr(d.err, ERR_TENSOR);
             // every copy issued has landed before the CTA may leave
             for (int s = 0; s < DW_SLOTS; ++s)
-                if ((used >> s) & 1u) mbar_wait(&full[s], (sw.fills(s) - 1) & 1, WAIT_NS);
+                if ((used >> s) & 1u) mbar_wait(&full[s], sw.last_fill(s), WAIT_NS);
         }
-    } else if (warp == 1) {
-        if (lane == 0) {                                      // MMA issuer
-            const uint32_t idesc = idesc_bf16(t.TNI);
-            SlotWalk sw;
-            bool ok = true;
+    } else if (warp == 1) {                                   // MMA issuer (lane 0)
+        const uint32_t idesc = idesc_bf16(t.TNI);
+        SlotWalk sw;
+        bool ok = true;
+        int lt = 0;
+        for (int tile = first; tile < end; tile += step, ++lt) {
+            read_marks(tile_m(tile));
+            if (lane != 0 || !ok) continue;
+            const int buf = lt & 1;
+            if (lt >= 2 && !(ok = mbar_wait(&acce[buf], ((lt >> 1) - 1) & 1, WAIT_NS))) continue;
+            fence_after();
+            const uint32_t accd = tmem + (uint32_t)buf * ncols;
             for (int it = 0; it < nk; ++it) {
                 const bool post = has_post(it);
                 const int s = sw.next(post);
-                if (!(ok = mbar_wait(&full[s], sw.fills(s) & 1, WAIT_NS))) break;
+                if (!(ok = mbar_wait(&full[s], sw.next_fill(s), WAIT_NS))) break;
                 fence_after();
                 const uint32_t xq = su32(smem + s * SLOT), sit = xq + t.NXQ * TILE_BYTES;
                 const uint32_t sp = sit + BTI, xp = sp + TILE_BYTES;
@@ -682,12 +741,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
                     uint32_t acc = it | k;
                     if (post)
                         for (int p = 0; p < t.NXP; ++p) {     // potentiation: SPOST . XPRE_p
-                            mma_bf16(tmem, sdesc(sp) + (uint64_t)(2 * k), sdesc(xp + p * BTI) + (uint64_t)(2 * k),
+                            mma_bf16(accd, sdesc(sp) + (uint64_t)(2 * k), sdesc(xp + p * BTI) + (uint64_t)(2 * k),
                                      idesc, acc != 0 ? 1u : 0u);
                             acc = 1u;
                         }
                     for (int q = 0; q < t.NXQ; ++q) {         // depression: XPOST_q . SINT
-                        mma_bf16(tmem, sdesc(xq + q * TILE_BYTES) + (uint64_t)(2 * k), sdesc(sit) + (uint64_t)(2 * k),
+                        mma_bf16(accd, sdesc(xq + q * TILE_BYTES) + (uint64_t)(2 * k), sdesc(sit) + (uint64_t)(2 * k),
                                  idesc, acc != 0 ? 1u : 0u);
                         acc = 1u;
                     }
@@ -696,28 +755,35 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
                 if (post) mma_commit(&empty[s + 1]);
                 sw.take(s, post);
             }
-            if (ok) mma_commit(accf);
-            else atomicOr(d.err, ERR_TENSOR);
+            if (ok) mma_commit(&accf[buf]);
+        }
+        if (lane == 0) {
+            if (!ok) atomicOr(d.err, ERR_TENSOR);
             mma_commit(drain);
             if (!mbar_wait(drain, 0, WAIT_NS)) atomicOr(d.err, ERR_TENSOR);
         }
     } else {                                                  // epilogue, part 1
-        if (ch0 < nch) wchunk_load(c, d, j, tn * t.TNI + ch0 * 16, wc);   // in flight during the product
-        if (tn == 0 && ks == 0 && half == 0 && j < c.N) {    // theta of the neuron (independent of W)
-            const int n = (int)t.colcnt[j];
-            double rr;
-            if (c.reduce == SNN_REDUCE_SUM) rr = (double)n;
-            else rr = c.B_pow2 ? __dmul_rn((double)n, (double)c.inv_B) : __ddiv_rn((double)n, (double)c.B);
-            d.theta[j] = __dadd_rn(__dmul_rn(d.theta[j], c.a_th), __dmul_rn(c.theta_plus, rr));
-            t.colcnt[j] = 0u;
-        }
-        const bool got = __all_sync(FULL, mbar_wait(accf, 0, WAIT_NS) ? 1 : 0) != 0;
-        if (!got) {
-            if (lane == 0) atomicOr(d.err, ERR_TENSOR);
-        } else {
+        int lt = 0;
+        for (int tile = first; tile < end; tile += step, ++lt) {
+            const int tm = tile_m(tile), tn = tile_n(tile), buf = lt & 1;
+            const int j = tm * 128 + row;
+            if (ch0 < nch) wchunk_load(c, d, j, tn * t.TNI + ch0 * 16, wc);   // in flight during the product
+            if (tn == 0 && ks == 0 && half == 0 && j < c.N) { // theta of the neuron (independent of W)
+                const int n = (int)t.colcnt[j];
+                double rr;
+                if (c.reduce == SNN_REDUCE_SUM) rr = (double)n;
+                else rr = c.B_pow2 ? __dmul_rn((double)n, (double)c.inv_B) : __ddiv_rn((double)n, (double)c.B);
+                d.theta[j] = __dadd_rn(__dmul_rn(d.theta[j], c.a_th), __dmul_rn(c.theta_plus, rr));
+                t.colcnt[j] = 0u;
+            }
+            const bool got = __all_sync(FULL, mbar_wait(&accf[buf], (lt >> 1) & 1, WAIT_NS) ? 1 : 0) != 0;
+            if (!got) {
+                if (lane == 0) atomicOr(d.err, ERR_TENSOR);
+                break;
+            }
             fence_after();
-            const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16);
-            if (t.KS == 1) {                                  // the update from the accumulator
+            const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * ncols;
+            if (!SLICED) {                                    // the update from the accumulator
                 for (int ch = ch0; ch < nch; ch += chs) {
                     uint32_t r[16];
                     tmem_ld16(tbase + (uint32_t)(ch * 16), r);
@@ -728,6 +794,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
                     if (i0 < c.n_in) wchunk_update(c, d, t, j, i0, D, wc);
                     if (ch + chs < nch) wchunk_load(c, d, j, tn * t.TNI + (ch + chs) * 16, wc);
                 }
+                fence_before();                               // this warp is done with the accumulator
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acce[buf]);
             } else {                                          // the partial tile for the cluster;
                 // every MMA has completed and every load was consumed, so the
                 // stage memory is free
@@ -746,9 +815,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
     }
     fence_before();
     __syncthreads();                                          // every partial tile of this CTA written
-    if (t.KS > 1) {
+    if (SLICED) {
         cluster_sync();                                       // ... and of every CTA of the cluster
         if (warp >= 2) {                                      // epilogue, part 2: slices in order
+            const int tm = blockIdx.x, tn = blockIdx.y, j = tm * 128 + row;
             const uint32_t prow = su32(smem) + (uint32_t)(row * PS) * 4u;
             for (int ch = ch0; ch < nch; ch += chs) {
                 float D[16];
@@ -779,7 +849,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
     }
     if (warp == 1) {
         fence_after();
-        tmem_free(tmem, ncols);
+        tmem_free(tmem, 2 * ncols);
     }
 }
 
@@ -855,6 +925,7 @@ TBufs tensor_plan(const Consts& c, int dense, int sms) {
     if (ks > nkb) ks = nkb;
     if (ks > DW_KSMAX) ks = DW_KSMAX;             // clusters of at most four slices
     t.KS = ks;
+    t.sms = sms;
     t.dense = dense;
     return t;
 }
@@ -901,7 +972,7 @@ cudaError_t launch_tensor_begin(const Consts& c, const Bufs& d, const TBufs& t, 
 // Dynamic shared memory of the two products at their largest tiles (three W
 // terms and 128 samples; three A tiles and four B tiles of 128 inputs): set
 // once per device, under a lock shared by every host thread.
-constexpr int CUR_SMEM_MAX = CUR_STAGES * (3 * TILE_BYTES + 128 * 128) + 1024 + 64;
+constexpr int CUR_SMEM_MAX = CUR_STAGES * (3 * TILE_BYTES + 128 * 128) + 1024 + 128;
 constexpr int DW_SMEM_MAX = DW_SLOTS * (4 * TILE_BYTES + 3 * 128 * 128) / 2 + 1024 + 128;
 static_assert(DW_SMEM_MAX <= 232448 && CUR_SMEM_MAX <= 232448, "227 KB of shared memory per CTA");
 
@@ -914,8 +985,10 @@ cudaError_t ensure_attributes() {
     std::lock_guard<std::mutex> lock(mu);
     if (!done[dev]) {
         TT_TRY(cudaFuncSetAttribute(k_t_current, cudaFuncAttributeMaxDynamicSharedMemorySize, CUR_SMEM_MAX));
-        TT_TRY(cudaFuncSetAttribute(k_t_dw<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM_MAX));
-        TT_TRY(cudaFuncSetAttribute(k_t_dw<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM_MAX));
+        TT_TRY(cudaFuncSetAttribute(k_t_dw<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM_MAX));
+        TT_TRY(cudaFuncSetAttribute(k_t_dw<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM_MAX));
+        TT_TRY(cudaFuncSetAttribute(k_t_dw<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM_MAX));
+        TT_TRY(cudaFuncSetAttribute(k_t_dw<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM_MAX));
         done[dev] = true;
     }
     return cudaSuccess;
@@ -931,9 +1004,9 @@ cudaError_t launch_tensor_step(const Consts& c, const Bufs& d, const TBufs& t, i
     TT_TRY(prof_stop(prof, s));
     TT_TRY(prof_start(prof, SNN_KERNEL_NEURON, s));
     if (t.dense) {
-        const size_t sm = (size_t)CUR_STAGES * cur_stage_bytes(t) + 1024 + 64;
-        k_t_current<<<dim3(t.Np / 128, (c.B + t.TB - 1) / t.TB), TC_THREADS, sm, s>>>(t.m_wt, t.m_sin, c, d, t,
-                                                                                    t_local);
+        const size_t sm = (size_t)CUR_STAGES * cur_stage_bytes(t) + 1024 + 128;
+        const int tiles = (t.Np / 128) * ((c.B + t.TB - 1) / t.TB);
+        k_t_current<<<tiles < t.sms ? tiles : t.sms, TC_THREADS, sm, s>>>(t.m_wt, t.m_sin, c, d, t, t_local);
     } else {
         k_t_gcurrent<<<dim3(t.Np / 128, (c.B + 15) / 16), 128, 0, s>>>(c, d, t, t_local);
     }
@@ -942,7 +1015,8 @@ cudaError_t launch_tensor_step(const Consts& c, const Bufs& d, const TBufs& t, i
     if (c.learn) {
         TT_TRY(prof_start(prof, SNN_KERNEL_STDP, s));
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(t.Np / 128, t.nti, t.KS);
+        const int tiles = (t.Np / 128) * t.nti;
+        cfg.gridDim = t.KS == 1 ? dim3(tiles < t.sms ? tiles : t.sms) : dim3(t.Np / 128, t.nti, t.KS);
         cfg.blockDim = dim3(TC_THREADS);
         cfg.dynamicSmemBytes = (size_t)DW_SLOTS * dw_slot_bytes(t) + 1024 + 128;
         cfg.stream = s;
@@ -953,8 +1027,9 @@ cudaError_t launch_tensor_step(const Consts& c, const Bufs& d, const TBufs& t, i
         at[0].val.clusterDim.z = (unsigned)t.KS;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        if (c.wmaster) TT_TRY(cudaLaunchKernelEx(&cfg, k_t_dw<true>, t.m_spost, t.m_xpost, t.m_xpre, t.m_sint, c, d, t, t_local));
-        else TT_TRY(cudaLaunchKernelEx(&cfg, k_t_dw<false>, t.m_spost, t.m_xpost, t.m_xpre, t.m_sint, c, d, t, t_local));
+        auto kern = c.wmaster ? (t.KS > 1 ? k_t_dw<true, true> : k_t_dw<true, false>)
+                              : (t.KS > 1 ? k_t_dw<false, true> : k_t_dw<false, false>);
+        TT_TRY(cudaLaunchKernelEx(&cfg, kern, t.m_spost, t.m_xpost, t.m_xpre, t.m_sint, c, d, t, t_local));
         TT_TRY(prof_stop(prof, s));
     }
     return cudaSuccess;
