@@ -26,6 +26,13 @@
 //   grid barrier.
 // The arithmetic is the per-step kernels' (same intrinsics, same order), so the
 // three run modes give bit-identical results.
+//
+// Loops are not unrolled unless that is written out or they are the separate
+// neuron passes' and the quiet-column pass's: the step's code does not fit the
+// instruction cache (92 % of its requests hit at 784->6400, 74 % at 784->100 with
+// the post-triggered rule), and unrolled it was half as large again.  784->6400, B =
+// 256: 7.05 ms a presentation unrolled, 6.82 so; 784->400, B = 1024: 8.58, 8.53;
+// the separate passes' loops are faster unrolled (784->100, B = 64: 3.07 and 3.52).
 #include <cfloat>
 #include <mutex>
 
@@ -234,6 +241,7 @@ __device__ __forceinline__ void encode_words(const Consts& c, const Bufs& d, con
     const int units = nmy * c.Iw;
     // a warp takes two (sample, 32-input word) units per pass: the loads of
     // both are issued before either draw is used
+#pragma unroll 1
     for (int u0 = warp; u0 < units; u0 += 2 * (PT / 32)) {
         int rr[2], iws[2], bs[2];
         bool on[2];
@@ -289,20 +297,24 @@ __device__ __forceinline__ void encode_lists(const Consts& c, const Bufs& d, con
     const int cur = (int)(tt & 1ull);
     const uint32_t* wbuf = (const uint32_t*)(sm + L.o_wbuf);
     const int nmy = cta < c.B ? (c.B - cta + L.G - 1) / L.G : 0;
+#pragma unroll 1
     for (int r = warp; r < nmy; r += PT / 32) {       // one warp per sample
         const int b = cta + L.G * r;
         uint16_t* out = d.act_idx + ((size_t)cur * c.B + b) * c.n_in;
         uint32_t running = 0;
+#pragma unroll 1
         for (int w0 = 0; w0 < c.Iw; w0 += 32) {
             const int w = w0 + lane;
             uint32_t word = w < c.Iw ? wbuf[r * c.Iw + w] : 0u;
             const uint32_t n = __popc(word);
             uint32_t incl = n;
+#pragma unroll 1
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y = __shfl_up_sync(FULL, incl, o);
                 if (lane >= o) incl += y;
             }
             uint32_t off = running + incl - n;
+#pragma unroll 1
             while (word) {
                 const int bit = __ffs(word) - 1;
                 word &= word - 1;
@@ -328,6 +340,7 @@ __device__ __forceinline__ void encode_phase(const Consts& c, const Bufs& d, con
 __device__ __forceinline__ void list_post_columns(const uint32_t* Qm, int nc, int Bw, uint32_t* nzQ,
                                                   uint32_t* nzQw, int* pcol, int* npc_out, int lane) {
     int npc = 0;
+#pragma unroll 1
     for (int jl0 = 0; jl0 < nc; jl0 += 32) {
         const int jl = jl0 + lane;
         int n = 0;
@@ -645,6 +658,7 @@ __device__ __noinline__ void depress_quiet_rows(
 #pragma unroll
     for (int m = 0; m < QPL; ++m) anyq = anyq || any[m];
     if (!__any_sync(FULL, anyq)) return;
+#pragma unroll 1
     for (int i0 = R * warp; i0 < NI; i0 += R * NW) {
         const int i = i0 + r;
         if (!on || i >= NI) continue;
@@ -655,6 +669,7 @@ __device__ __noinline__ void depress_quiet_rows(
         if (LISTS) {
             int e0, e1;
             row_span(offs, i, e0, e1);
+#pragma unroll 1
             for (int e = e0; e < e1; ++e) {
                 const float* er = Es + (int)lst[e] * nst + 4 * l;
 #pragma unroll
@@ -671,6 +686,7 @@ __device__ __noinline__ void depress_quiet_rows(
         } else {   // the row's spike words, its nonzero words only, ascending b
             const uint32_t* Pi = preS + i * PS;
             uint32_t words = Bw <= 32 ? nzP[i] : 0xFFFFFFFFu;
+#pragma unroll 1
             for (int w = 0; w < Bw; ++w) {
                 if (Bw <= 32) {
                     if (!words) break;
@@ -678,6 +694,7 @@ __device__ __noinline__ void depress_quiet_rows(
                     words &= words - 1;
                 }
                 uint32_t mk = Pi[w];
+#pragma unroll 1
                 while (mk) {
                     const float* er = Es + (w * 32 + __ffs(mk) - 1) * nst + 4 * l;
                     mk &= mk - 1;
@@ -765,6 +782,7 @@ __device__ __noinline__ void update_post_column_groups(
         const int* pcol, bool lists, const int* offs, const uint16_t* lst, const uint32_t* preS, int PS,
         const uint32_t* nzP, const float* xpre, int npc, int NI, int nc, int nst, int Bw, int warp, int lane) {
     const int nch = (NI + 31) / 32, ngr = (npc + PG - 1) / PG;
+#pragma unroll 1
     for (int u = warp; u < ngr * nch; u += NW) {
         const int k0 = (u / nch) * PG, kn = min(PG, npc - k0);
         const int* pc = pcol + k0;
@@ -777,11 +795,13 @@ __device__ __noinline__ void update_post_column_groups(
         uint32_t un = 0u, cw[PG];
 #pragma unroll
         for (int k = 0; k < PG; ++k) un |= k < kn ? Qm[pc[k]] : 0u;
+#pragma unroll 1
         for (;;) {
             int bs[XC];
             int n = 0;
 #pragma unroll
             for (int z = 0; z < XC; ++z) {
+#pragma unroll 1
                 while (un == 0u && w + 1 < Bw) {
                     ++w;
 #pragma unroll
@@ -828,6 +848,7 @@ __device__ __noinline__ void update_post_column_groups(
         if (c.dep_on && lists) {   // every input-spike sample (e is 0 where j has not fired)
             int e0, e1;
             row_span(offs, i, e0, e1);
+#pragma unroll 1
             for (int e = e0; e < e1; ++e) {
                 const float* er = Es + (int)lst[e] * nst;
 #pragma unroll
@@ -837,6 +858,7 @@ __device__ __noinline__ void update_post_column_groups(
                                  // in which a column of the group has fired (e is 0 elsewhere)
             const uint32_t* Pi = preS + i * PS;
             uint32_t words = Bw <= 32 ? nzP[i] : 0xFFFFFFFFu;
+#pragma unroll 1
             for (int ww = 0; ww < Bw; ++ww) {
                 if (Bw <= 32) {
                     if (!words) break;
@@ -847,6 +869,7 @@ __device__ __noinline__ void update_post_column_groups(
 #pragma unroll
                 for (int k = 0; k < PG; ++k) fired |= k < kn ? Sm[ww * nc + jls[k]] : 0u;
                 uint32_t m = Pi[ww] & fired;
+#pragma unroll 1
                 while (m) {
                     const float* er = Es + (ww * 32 + __ffs(m) - 1) * nst;
                     m &= m - 1;
@@ -1105,6 +1128,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
     const int B = c.B, N = c.N, NI = c.n_in;
     const Units U = units_of(B, nc);
     int b = threadIdx.x / U.nq, qd = threadIdx.x % U.nq;
+#pragma unroll 1
     for (int sl = 0; sl < U.nslot; ++sl, unit_next(U, b, qd)) {
         {
             const int j = 4 * qd;
@@ -1121,6 +1145,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
                     // the staged entries two at a time (both weight rows in flight,
                     // the sums in order), then any beyond them from global memory
                     int a = 0;
+#pragma unroll 1
                     for (; a + 1 < ns; a += 2) {
                         const float4 w = *(const float4*)(wc + (int)al[a] * nst);
                         const float4 v = *(const float4*)(wc + (int)al[a + 1] * nst);
@@ -1129,6 +1154,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
                         I2 = __fadd_rn(__fadd_rn(I2, w.z), v.z);
                         I3 = __fadd_rn(__fadd_rn(I3, w.w), v.w);
                     }
+#pragma unroll 1
                     for (; a < na; ++a) {
                         const int r = a < ns ? (int)al[a] : (int)__ldcg(&ag[a]);
                         const float4 w = *(const float4*)(wc + r * nst);
@@ -1139,6 +1165,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
                     }
                 } else if (c.wprec == SNN_W_BF16) {
                     int a = 0;
+#pragma unroll 1
                     for (; a + 1 < ns; a += 2) {
                         const float4 w = *(const float4*)(wc + (int)al[a] * nst);
                         const float4 v = *(const float4*)(wc + (int)al[a + 1] * nst);
@@ -1147,6 +1174,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
                         I2 = __fadd_rn(__fadd_rn(I2, w_read_bf16(w.z)), w_read_bf16(v.z));
                         I3 = __fadd_rn(__fadd_rn(I3, w_read_bf16(w.w)), w_read_bf16(v.w));
                     }
+#pragma unroll 1
                     for (; a < na; ++a) {
                         const int r = a < ns ? (int)al[a] : (int)__ldcg(&ag[a]);
                         const float4 w = *(const float4*)(wc + r * nst);
@@ -1161,6 +1189,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
                     const float v0 = inv[j], v1 = j + 1 < nc ? inv[j + 1] : 1.0f;
                     const float v2 = j + 2 < nc ? inv[j + 2] : 1.0f, v3 = j + 3 < nc ? inv[j + 3] : 1.0f;
                     int a = 0;
+#pragma unroll 1
                     for (; a + 1 < ns; a += 2) {
                         const float4 w = *(const float4*)(wc + (int)al[a] * nst);
                         const float4 u = *(const float4*)(wc + (int)al[a + 1] * nst);
@@ -1169,6 +1198,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
                         I2 = __fadd_rn(__fadd_rn(I2, w_read_e4m3(w.z, v2)), w_read_e4m3(u.z, v2));
                         I3 = __fadd_rn(__fadd_rn(I3, w_read_e4m3(w.w, v3)), w_read_e4m3(u.w, v3));
                     }
+#pragma unroll 1
                     for (; a < na; ++a) {
                         const int r = a < ns ? (int)al[a] : (int)__ldcg(&ag[a]);
                         const float4 w = *(const float4*)(wc + r * nst);
@@ -1305,16 +1335,20 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
     const unsigned long long base = d.step[0];
 
     // ---- the CTA's columns: weights (padding columns 0), masks, thresholds
+#pragma unroll 1
     for (int k = tid; k < NI * nst; k += PT) {
         const int i = k / nst, jl = k % nst;
         Ws[k] = jl < nc ? d.W[(size_t)i * N + j0 + jl] : 0.0f;
         if (WLs) WLs[k] = jl < nc ? d.W_lo[(size_t)i * N + j0 + jl] : 0.0f;
     }
+#pragma unroll 1
     for (int k = tid; k < B * nst; k += PT) Es[k] = 0.0f;
+#pragma unroll 1
     for (int k = tid; k < Bw * nc; k += PT) {
         const int w = k / nc, jl = k % nc;
         Sm[k] = d.spkT[(size_t)(j0 + jl) * Bw + w];
     }
+#pragma unroll 1
     for (int jl = tid; jl < nc; jl += PT) thS[jl] = d.theta[j0 + jl];
 
     // ---- neuron state of the CTA's units into tensor memory
@@ -1335,6 +1369,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
         tq = s_tmem + ((uint32_t)(32 * ((tid >> 5) & 3)) << 16) + (uint32_t)((tid >> 7) * QT * 4);
         if (FUSED) {
             int b = tid / U.nq, qd = tid % U.nq;
+#pragma unroll 1
             for (int sl = 0; sl < U.nslot; ++sl, unit_next(U, b, qd)) {
                 const int j = 4 * qd;
                 uint32_t r[16];
@@ -1354,6 +1389,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             }
         } else {
             int b = tid / nc, jl = tid % nc;
+#pragma unroll 1
             for (int q = 0; q < QN; ++q) {
                 Item it{0.0f, 0.0f, 0.0f, 0u};
                 if (tid + q * PT < BN) {
@@ -1375,6 +1411,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
 
     // ---- prologue: input spikes of the first step
     if (cta == 0)
+#pragma unroll 1
         for (int b = tid; b < B; b += PT) d.cnt[(size_t)(base % 3ull) * B + b] = 0u;
     encode_phase(c, d, L, sm, base, 0);
     if (tid == 0) s_lovf[0] = s_lany[0] = 0;
@@ -1384,6 +1421,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
     bool ok = grid_wait(bar, d.err, G * nbar + (c.test_timeout ? 1u : 0u),
                         c.test_timeout ? TEST_SPIN_LIMIT : SPIN_LIMIT);
 
+#pragma unroll 1
     for (int t = 0; t < T && ok; ++t) {
         const unsigned long long tt = base + (unsigned long long)t;
         const int cur = (int)(tt & 1ull), p3 = (int)(tt % 3ull);
@@ -1397,6 +1435,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
         if (L.amask) {   // the step's masks for the STDP phase: chunk k of 8 per row,
                          // from the thread that reads it back there
             uint32_t* preA = (uint32_t*)(sm + L.o_pres);
+#pragma unroll 1
             for (int k = tid; k < NI * 8; k += PT)
                 cp_async16(preA + (k >> 3) * L.ps + 4 * (k & 7), pre_src + 4 * k);
             cp_async_commit();
@@ -1423,17 +1462,21 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
         uint4 av0 = make_uint4(0u, 0u, 0u, 0u);
         if (acts_vec && tid < acts_n)
             av0 = __ldcg((const uint4*)(acts_src + (size_t)(tid / acts_per) * NI) + (tid % acts_per));
+#pragma unroll 1
         for (int k = tid; k < Bw * nc; k += PT) Qm[k] = 0u;
+#pragma unroll 1
         for (int jl = tid; jl < nc; jl += PT) {   // thresholds after the previous step's STDP
             if (c.learn && t > 0) thS[jl] = theta_next(c, thS[jl], (int)nzQ[jl]);
             thj[jl] = __fadd_rn(c.e_thresh, __double2float_rn(thS[jl]));
         }
         if (cta == 0)   // accumulator of the next step (its last reader was step tt-1)
+#pragma unroll 1
             for (int b = tid; b < B; b += PT) d.cnt[(size_t)((p3 + 1) % 3) * B + b] = 0u;
         {   // input-major masks of step tt+2, slot of step tt-2: every CTA has run
             // that step's STDP before signalling its encode of step tt
             const size_t n_pre = (size_t)NI * Bw;
             uint32_t* z = d.preT + (size_t)((tt + 2ull) % PRET_SLOTS) * n_pre;
+#pragma unroll 1
             for (size_t k = (size_t)cta * PT + tid; k < n_pre; k += (size_t)G * PT) z[k] = 0u;
         }
         // the previous step's inhibitory counts and this step's active-input counts
@@ -1441,6 +1484,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             cntS[tid] = cn0;
             actN[tid] = an0;
         }
+#pragma unroll 1
         for (int b = tid + PT; b < B; b += PT) {
             cntS[b] = __ldcg(&cnt_src[b]);
             actN[b] = __ldcg(&actn_src[b]);
@@ -1448,6 +1492,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
         // first entries of every sample's active-input list (in bounds: caps <= n_in)
         if (acts_vec) {
             if (tid < acts_n) ((uint4*)actS)[tid] = av0;
+#pragma unroll 1
             for (int k0 = tid + PT; k0 < acts_n; k0 += 2 * PT) {
                 uint4 v4[2];
 #pragma unroll
@@ -1463,6 +1508,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             }
         } else {
             const int n = B * caps;
+#pragma unroll 1
             for (int k = tid; k < n; k += PT)
                 actS[(k / caps) * CAPS + (k % caps)] = __ldcg(&acts_src[(size_t)(k / caps) * NI + (k % caps)]);
         }
@@ -1481,6 +1527,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             const int nwr = NI < PT ? (NI + 31) / 32 : NW;   // warps with rows
             const int capw = L.lcap / nwr, reg0 = wp * capw;
             int run = 0;                                     // the warp's entries so far
+#pragma unroll 1
             for (int r0 = 0; r0 < NI; r0 += PT) {
                 const int i = r0 + tid;
                 uint32_t wr[8];                              // the row's words
@@ -1523,6 +1570,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
 #pragma unroll
                             for (int w = 0; w < 8; ++w) {
                                 uint32_t m = w < Bw ? wr[w] : 0u;
+#pragma unroll 1
                                 while (m) {
                                     lst[q++] = (uint16_t)(w * 32 + __ffs(m) - 1);
                                     m &= m - 1;
@@ -1546,9 +1594,12 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
         if (t + 1 < T) encode_words(c, d, L, sm, tt + 1, t + 1);
         if (c.wprec == SNN_W_FP8E4M3) {   // column scales of this step's weights
             const int warp = tid >> 5, lane = tid & 31;
+#pragma unroll 1
             for (int jl = warp; jl < nc; jl += NW) {
                 float m = 0.0f;
+#pragma unroll 1
                 for (int i = lane; i < NI; i += 32) m = fmaxf(m, fabsf(Ws[i * nst + jl]));
+#pragma unroll 1
                 for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
                 if (lane == 0) {
                     const float sc = e4m3_scale_of(m);
@@ -1599,6 +1650,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                              // read back, each row's nonzero words from the 8 lanes of its row
                 cp_async_wait_all();
                 const int nch = NI * 8;
+#pragma unroll 1
                 for (int k0 = tid - (tid & 31); k0 < nch; k0 += PT) {
                     const int k = k0 + (tid & 31);
                     uint32_t nz = 0u;
@@ -1615,10 +1667,12 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             } else if (L.masks) {   // the step's masks, padded rows, and each row's nonzero words:
                              // a thread per row, its words in 16-byte loads issued together
                 const uint32_t* src = d.preT + (size_t)(tt % PRET_SLOTS) * NI * Bw;
+#pragma unroll 1
                 for (int i = tid; i < NI; i += PT) {
                     const uint32_t* row = src + (size_t)i * Bw;
                     uint32_t nz = 0u;
                     if ((Bw & 3) == 0) {
+#pragma unroll 1
                         for (int w0 = 0; w0 < Bw; w0 += 16) {
                             uint4 q[4];
 #pragma unroll
@@ -1638,6 +1692,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                             }
                         }
                     } else {
+#pragma unroll 1
                         for (int w = 0; w < Bw; ++w) {
                             const uint32_t m = __ldcg(&row[w]);
                             preS[i * PS + w] = m;
@@ -1648,6 +1703,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                 }
             } else if (c.reduce == SNN_REDUCE_MAX || !lists) {   // the step's masks, padded rows
                 const uint32_t* src = d.preT + (size_t)(tt % PRET_SLOTS) * NI * Bw;
+#pragma unroll 1
                 for (int k = tid; k < NI * Bw; k += PT) preS[(k / Bw) * PS + (k % Bw)] = __ldcg(&src[k]);
             }
             if (!early) __syncthreads();
@@ -1657,6 +1713,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             //     rule has none; it clips every weight, and a column scaled to its
             //     weight sum may have left the bounds)
             if (c.rule == SNN_RULE_POST_NORM) {
+#pragma unroll 1
                 for (int k = tid; k < NI * nc; k += PT) {
                     const int i = k / nc, jl = k % nc;
                     if (nzQ[jl] == 0u) Ws[i * nst + jl] = fminf(fmaxf(Ws[i * nst + jl], c.w_min), c.w_max);
@@ -1697,6 +1754,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                 // post-spiking samples, the same for every lane, XC at a time with
                 // their x_pre loads issued together; depression over the lane's own
                 // (input spike and neuron-has-fired) samples.
+#pragma unroll 1
                 for (int u = warp; u < (grouped ? 0 : ntask); u += NW) {
                     const int jl = pcol[u / nch];
                     const int i = (u % nch) * 32 + lane;
@@ -1707,11 +1765,13 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                     int nev = 0;
                     int w = 0;
                     uint32_t qb = Qm[jl];
+#pragma unroll 1
                     for (;;) {
                         int bs[XC];
                         int n = 0;
 #pragma unroll
                         for (int z = 0; z < XC; ++z) {
+#pragma unroll 1
                             while (qb == 0u && w + 1 < Bw) qb = Qm[++w * nc + jl];
                             bs[z] = -1;
                             if (qb) {
@@ -1748,6 +1808,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                     if (lists && dep_on) {   // every input-spike sample (e is 0 where j has not fired)
                         int e0, e1;
                         row_span(offs, i, e0, e1);
+#pragma unroll 1
                         for (int e = e0; e < e1; ++e) {
                             const int b = lst[e];
                             if (is_max && ((Qm[(b >> 5) * nc + jl] >> (b & 31)) & 1u)) continue;
@@ -1757,6 +1818,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                         }
                     }
                     uint32_t words = lists ? 0u : (Bw <= 32 ? nzP[i] : 0xFFFFFFFFu);
+#pragma unroll 1
                     for (int ww = 0; ww < (lists || !dep_on ? 0 : Bw); ++ww) {
                         if (Bw <= 32) {
                             if (!words) break;
@@ -1765,6 +1827,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                         }
                         uint32_t m = Pi[ww] & Sm[ww * nc + jl];
                         if (is_max) m &= ~Qm[ww * nc + jl];     // post samples were handled above
+#pragma unroll 1
                         while (m) {
                             const int bit = __ffs(m) - 1;
                             m &= m - 1;
@@ -1790,13 +1853,41 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                 __syncthreads();
                 float* nrm = (float*)(sm + L.o_nrm);
                 const int npc = s_nq;
+#pragma unroll 1
                 for (int u = tid; u < npc; u += PT) {
-                    const int jl = pcol[u];
-                    float S = 0.0f;
-                    for (int i = 0; i < NI; ++i) S = __fadd_rn(S, Ws[i * nst + jl]);
+                    // one chain of adds, sixteen loads ahead of it (narrow layers:
+                    // rows of four floats, so the loads take immediate offsets);
+                    // 784->100, B = 64, max: 3.44 -> 3.07 ms a presentation
+                    const int rs = NARROW ? 4 : nst;
+                    const float* wc = Ws + pcol[u];
+                    float S = 0.0f, wa[16], wb[16];
+                    auto load16 = [&](float (&w)[16], const float* p) {
+#pragma unroll
+                        for (int z = 0; z < 16; ++z) w[z] = p[z * rs];
+                    };
+                    auto add16 = [&](const float (&w)[16]) {
+#pragma unroll
+                        for (int z = 0; z < 16; ++z) S = __fadd_rn(S, w[z]);
+                    };
+                    int i = 0;
+                    if (NI >= 32) {
+                        load16(wa, wc);
+#pragma unroll 1
+                        for (; i + 48 <= NI; i += 32) {        // wa holds rows i .. i + 15
+                            load16(wb, wc + (i + 16) * rs);
+                            add16(wa);
+                            load16(wa, wc + (i + 32) * rs);
+                            add16(wb);
+                        }
+                        add16(wa);
+                        i += 16;
+                    }
+#pragma unroll 4
+                    for (; i < NI; ++i) S = __fadd_rn(S, wc[i * rs]);
                     nrm[u] = S == 0.0f ? 1.0f : __fdiv_rn(c.w_norm, S);   // S = 0: unchanged
                 }
                 __syncthreads();
+#pragma unroll 1
                 for (int k = tid; k < NI * npc; k += PT) {
                     const int i = k / npc, u = k % npc;
                     const int jl = pcol[u];
@@ -1813,6 +1904,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
 
     // ---- thresholds after the last step's STDP
     if (c.learn && T > 0)
+#pragma unroll 1
         for (int jl = tid; jl < nc; jl += PT) thS[jl] = theta_next(c, thS[jl], (int)nzQ[jl]);
 
     // ---- write the CTA's columns back, and the neuron state held in tensor memory
@@ -1820,6 +1912,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
     if (tstate) {
         if (FUSED) {
             int b = tid / U.nq, qd = tid % U.nq;
+#pragma unroll 1
             for (int sl = 0; sl < U.nslot; ++sl, unit_next(U, b, qd)) {
                 const int j = 4 * qd;
                 uint32_t r[16];
@@ -1838,6 +1931,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             }
         } else {
             int b = tid / nc, jl = tid % nc;
+#pragma unroll 1
             for (int q = 0; q < QN; ++q) {
                 Item it;
                 __syncwarp();
@@ -1863,13 +1957,16 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
         }
     }
     if (c.learn) {
+#pragma unroll 1
         for (int k = tid; k < NI * nc; k += PT) {
             const int i = k / nc, jl = k % nc;
             d.W[(size_t)i * N + j0 + jl] = Ws[i * nst + jl];
             if (WLs) d.W_lo[(size_t)i * N + j0 + jl] = WLs[i * nst + jl];
         }
+#pragma unroll 1
         for (int jl = tid; jl < nc; jl += PT) d.theta[j0 + jl] = thS[jl];
     }
+#pragma unroll 1
     for (int k = tid; k < Bw * nc; k += PT) {
         const int w = k / nc, jl = k % nc;
         d.spkT[(size_t)(j0 + jl) * Bw + w] = Sm[k];
