@@ -110,26 +110,55 @@ __host__ __device__ __forceinline__ size_t state_elems(int B, int N) { return (s
 constexpr uint16_t BF16_ONE = 0x3F80;
 
 // ---- dense form: tcgen05 GEMM with the neuron update in the epilogue -------
-constexpr int GBM = 128, GBN = 256, GBK = 64, GSTAGES = 4;
-constexpr int GA_BYTES = GBM * GBK * 2, GB_BYTES = GBN * GBK * 2, GSTAGE = GA_BYTES + GB_BYTES;
+// A pair of CTAs (a cluster on two neighbouring SMs) computes 256 samples x GBN
+// neurons with cta_group::2 products: each CTA stages its own 128 samples and half
+// of the neurons' weights, and keeps its samples' accumulator.
+constexpr int GBM = 128, GBN = 256, GBK = 64, GSTAGES = 6;
+constexpr int GWB = GBN / 2;             // weight rows of one TMA copy
+constexpr int GA_BYTES = GBM * GBK * 2, GW_BYTES = GWB * GBK * 2, GSTAGE = GA_BYTES + GBN / 2 * GBK * 2;
 constexpr int GSMEM = GSTAGES * GSTAGE + 1024 + 256;
 constexpr int GEPI_WARPS = 8, GTHREADS = 64 + 32 * GEPI_WARPS;
 constexpr unsigned long long GWAIT_NS = 2000000000ull;   // bounded waits: 2 s, then the error flag
-// instruction descriptor: FP32 accumulator, bfloat16 A and B, both K-major, M=128
-__host__ __device__ constexpr uint32_t gidesc(int n) { return snn::tc::idesc_bf16(n); }
-static_assert(GBM == 128, "the instruction descriptor is for M = 128");
+// instruction descriptor: FP32 accumulator, bfloat16 A and B, both K-major, M = 256
+// (the pair's samples)
+__host__ __device__ constexpr uint32_t gidesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(2 * GBM >> 4) << 24);
+}
 
-// Tiles of the dense form: ntn_drive neuron tiles of GBN columns per 128 samples,
-// then, when the readout is fused (n_out <= GBN), one readout tile whose
+// Work items of the dense form, item = pair + i * pairs: the drive tiles (nd of
+// them, ntn_drive neuron tiles of GBN columns per 256 samples, neuron tiles
+// fastest), the ones from nfull on cut into `parts` of GBN / parts columns, then,
+// when the readout is fused (n_out <= GBN), one readout item per 256 samples, whose
 // weight rows start at R0 = ntn_drive * GBN and whose MMAs are n_ro wide.
-// With enc_next, drive tile (tm, tn) also draws the next step's input spikes of
-// its samples for inputs [tn * a_per, (tn + 1) * a_per), a_per a multiple of 32.
+//
+// The cut tiles are the last round's, when it would leave pairs idle: `parts` is the
+// largest of 1, 2 and 4 whose items fill no second round.
+// Per step over 60 steps, whole tiles in a CTA / whole tiles in a pair / cut tiles in
+// a pair: 1024->4096, B = 4096 (28 of 256 tiles cut) 167 / 149 / 147 us; B = 256 (16
+// tiles, quarters) 45.2 / 47.3 / 41.0; 300->626, B = 626 (9 tiles, quarters: the
+// third neuron tile's ragged columns are 32 of one warp's instead of 64 or more) 81
+// / 83 / 25.5; 300->1000, B = 128 54 / 56 / 23.
+//
+// With enc_next, the items of drive tile (tm, tn) also draw the next step's input
+// spikes of its samples for inputs [tn * a_per, (tn + 1) * a_per), a_per a multiple
+// of 32.
 // Every step's spike words go to hist slot `slot`; to sh only with keep_sh (the
 // run's last step, or a readout launch of its own).
 struct DenseGeom {
-    int ntn_drive, ntn, ntiles, fused, n_ro, a_per, enc_next;
+    int ntn_drive, fused, n_ro, a_per, enc_next;
     int slot, keep_sh;
+    int nd, nfull, parts, nitems;
 };
+struct DenseItem {
+    int tmp, tn, part, width;   // pair's sample tile, neuron tile, which part of it, its columns
+    bool ro;
+};
+__device__ __forceinline__ DenseItem dense_item(const DenseGeom& g, int i) {
+    const int ncut = (g.nd - g.nfull) * g.parts, k = i - g.nfull;
+    if (k >= ncut) return {k - ncut, g.ntn_drive, 0, g.n_ro, true};
+    const int tile = k < 0 ? i : g.nfull + k / g.parts;
+    return {tile / g.ntn_drive, tile % g.ntn_drive, k < 0 ? 0 : k % g.parts, k < 0 ? GBN : GBN / g.parts, false};
+}
 constexpr int HIST = 31;                 // steps between two updates of the counts (five-bit counters)
 
 // waits for the phase with the given parity to complete; false after GWAIT_NS
@@ -677,8 +706,8 @@ __global__ void __launch_bounds__(256) k_rec_fold(RecConsts c, RecBufs d, int n)
                      ((k4 >> u) & 1u) << 4;
 }
 
-// Dense form, epilogue of one warp's half tile (32 samples x 128 neurons j0..,
-// all < N) as a 3-deep pipeline over 16-neuron steps: the state loads of steps
+// Dense form, epilogue of one warp's half item (32 samples x 16 * steps neurons
+// j0.., all < N; steps is EPH, EPH / 2 or EPH / 4) as a 3-deep pipeline over 16-neuron steps: the state loads of steps
 // k+1 and k+2 are in flight while step k is computed and stored, so the loads of
 // consecutive steps leave no gap.  The warp's accumulator is
 // released (acce) after its last tensor-memory load.  Each pipeline slot is a
@@ -699,15 +728,15 @@ __device__ __forceinline__ void epi_load(const RecConsts& c, const RecBufs& d, E
 
 template <int K>
 __device__ __forceinline__ void epi_step(const RecConsts& c, const RecBufs& d, const EpiSlot& sl, uint32_t tcol,
-                                         int b, bool live, int j0, int cur, int nxt, int t_local,
-                                         uint64_t* acce_bar, const DenseGeom& g, uint32_t& word) {
+                                         int b, bool live, int j0, int steps, int cur, int nxt, int t_local,
+                                         uint32_t acce_bar, const DenseGeom& g, uint32_t& word) {
     const int lane = threadIdx.x & 31;
     uint32_t r[16];
     tmem_ld16(tcol + (uint32_t)(16 * K), r);
-    if (K == EPH - 1) {
+    if (K == EPH - 1 || ((K == EPH / 2 - 1 || K == EPH / 4 - 1) && K == steps - 1)) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(su32(acce_bar)) : "memory");
+        if (lane == 0) snn::tc::mbar_arrive_cluster(acce_bar);
     }
     uint32_t w16 = 0u;
     if (live) {
@@ -740,39 +769,48 @@ __device__ __forceinline__ void epi_step(const RecConsts& c, const RecBufs& d, c
 // one pipeline iteration H: load step H (into slot H % EPD), then compute step H - (EPD - 1)
 template <int H>
 __device__ __forceinline__ void epi_iter(const RecConsts& c, const RecBufs& d, EpiSlot (&sl)[EPD], uint32_t tcol,
-                                         int b, bool live, int j0, int cur, int nxt, int t_local,
-                                         uint64_t* acce_bar, const DenseGeom& g, uint32_t& word) {
-    if (H < EPH && live) epi_load(c, d, sl[H % EPD], b, j0 + 16 * H);
+                                         int b, bool live, int j0, int steps, int cur, int nxt, int t_local,
+                                         uint32_t acce_bar, const DenseGeom& g, uint32_t& word) {
+    if (H < EPH && (H < EPH / 4 || H < steps) && live) epi_load(c, d, sl[H % EPD], b, j0 + 16 * H);
     if (H >= EPD - 1)
         epi_step<(H >= EPD - 1 ? H - (EPD - 1) : 0)>(c, d, sl[(H >= EPD - 1 ? H - (EPD - 1) : 0) % EPD], tcol, b, live,
-                                                     j0, cur, nxt, t_local, acce_bar, g, word);
+                                                     j0, steps, cur, nxt, t_local, acce_bar, g, word);
 }
 
 __device__ __forceinline__ void dense_epilogue_half_pipelined(const RecConsts& c, const RecBufs& d, uint32_t tcol,
-                                                              int b, bool live, int j0, int cur, int nxt,
-                                                              int t_local, uint64_t* acce_bar, const DenseGeom& g) {
+                                                              int b, bool live, int j0, int steps, int cur, int nxt,
+                                                              int t_local, uint32_t acce_bar, const DenseGeom& g) {
     static_assert(EPD == 3 && EPH == 8, "the iterations below are written out for these sizes");
     EpiSlot sl[EPD];
     uint32_t word = 0u;
-    epi_iter<0>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
-    epi_iter<1>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
-    epi_iter<2>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
-    epi_iter<3>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
-    epi_iter<4>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
-    epi_iter<5>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
-    epi_iter<6>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
-    epi_iter<7>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
-    epi_iter<8>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
-    epi_iter<9>(c, d, sl, tcol, b, live, j0, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<0>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<1>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<2>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<3>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
+    if (steps == EPH / 4) return;
+    epi_iter<4>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<5>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
+    if (steps == EPH / 2) return;
+    epi_iter<6>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<7>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<8>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
+    epi_iter<9>(c, d, sl, tcol, b, live, j0, steps, cur, nxt, t_local, acce_bar, g, word);
 }
 
-// Dense form, persistent: one CTA per SM walks the 128-sample x 256-neuron
-// tiles (tile = blockIdx.x + i * gridDim.x, neuron tiles fastest).  Warp 0
-// lane 0 streams the operand tiles with TMA through GSTAGES stages; warp 1
-// owns the tensor memory (two 256-column accumulators) and one lane issues
-// the MMAs; warps 2..9 run the epilogue of the previous tile while the next
-// one accumulates (warp w reads tensor-memory lanes 32*(w%4).., half
-// (w-2)/4 of the tile's columns).
+// Dense form, persistent: a pair of CTAs per two SMs walks the 256-sample x
+// 256-neuron tiles (tile = pair + i * pairs, neuron tiles fastest).  Warp 0 lane 0
+// of each CTA streams its operand tiles with TMA through GSTAGES stages, all bytes
+// of a stage counted on the first CTA's barrier; warp 1 owns the tensor memory (two
+// 256-column accumulators), and one lane of the first CTA issues the products of
+// both, whose commits reach the barriers of both; warps 2..9 run the epilogue of
+// the previous tile while the next one accumulates (warp w reads tensor-memory
+// lanes 32*(w%4).., half (w-2)/4 of the tile's columns, of its CTA's samples).
+//
+// The pair halves the weights' way into each SM: 32 KB of operands a stage instead
+// of 48, of which a CTA alone took 74 bytes a cycle: 1024->4096, B = 4096, a CTA
+// per tile took 157 us a step, the pair 140 (T = 500), and 1024->4096, B = 2304,
+// 117 and 97.  What is left above the products' own 512 cycles a stage is the
+// epilogue beside them.
 __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant__ CUtensorMap tmS0,
                                                            const __grid_constant__ CUtensorMap tmS1,
                                                            const __grid_constant__ CUtensorMap tmW,
@@ -780,26 +818,28 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
                                                            uint32_t* err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t* full = (uint64_t*)(smem + GSTAGES * GSTAGE);
+    uint64_t* full = (uint64_t*)(smem + GSTAGES * GSTAGE);   // (the first CTA's: both CTAs' bytes)
     uint64_t* empty = full + GSTAGES;
     uint64_t* accf = empty + GSTAGES;      // [2] accumulator ready (MMA commit)
-    uint64_t* acce = accf + 2;             // [2] accumulator drained (epilogue warps)
+    uint64_t* acce = accf + 2;             // [2] accumulator drained (the first CTA's: both CTAs' epilogue warps)
     uint64_t* drain = acce + 2;            // the MMA thread's last commit
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)(blockIdx.x & 1u), pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
     if (tid == 0) {
         for (int s = 0; s < GSTAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&accf[i], 1); mbar_init(&acce[i], GEPI_WARPS); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&accf[i], 1); mbar_init(&acce[i], 2 * GEPI_WARPS); }
         mbar_init(drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+    if (warp == 1) {                       // (both CTAs of the pair)
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
                      :: "r"(su32(&s_tmem)), "r"(2 * GBN) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    snn::tc::cluster_sync();               // both CTAs' barriers and tensor memory are ready
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s_tmem;
     const int nk = d.K / GBK;
@@ -810,30 +850,36 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
         if (lane == 0) {                                  // TMA producer
             int it = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < g.ntiles && ok; tile += gridDim.x) {
-                const int tm = tile / g.ntn, tn = tile % g.ntn;
+            for (int i = pair; i < g.nitems && ok; i += pairs) {
+                const DenseItem w = dense_item(g, i);
+                const int tm = 2 * w.tmp + rank, rows = w.width / 2;   // this CTA's half of the weights
+                const int wrow = w.tn * GBN + w.part * w.width + rank * rows, copies = (rows + GWB - 1) / GWB;
                 for (int kb = 0; kb < nk; ++kb, ++it) {
                     const int s = it % GSTAGES, round = it / GSTAGES;
                     if (it >= GSTAGES && !(ok = mbar_wait(&empty[s], (round - 1) & 1))) break;
                     uint8_t* st = smem + s * GSTAGE;
-                    mbar_expect_tx(&full[s], GSTAGE);
-                    tma_2d(st, tmS, kb * GBK, tm * GBM, &full[s]);
-                    tma_2d(st + GA_BYTES, &tmW, kb * GBK, tn * GBN, &full[s]);
+                    const uint32_t f = snn::tc::cluster_map(su32(&full[s]), 0u);
+                    if (rank == 0) mbar_expect_tx(&full[s], 2 * (GA_BYTES + copies * GW_BYTES));
+                    snn::tc::tma_2d_pair(st, tmS, kb * GBK, tm * GBM, f);
+                    for (int q = 0; q < copies; ++q)
+                        snn::tc::tma_2d_pair(st + GA_BYTES + q * GW_BYTES, &tmW, kb * GBK, wrow + q * GWB, f);
                 }
             }
+            // the commits that free the last stages arrive here from the first CTA:
+            // this one stays until they have
+            for (int j = max(0, it - GSTAGES); j < it && ok; ++j) ok = mbar_wait(&empty[j % GSTAGES], (j / GSTAGES) & 1);
             if (!ok) atomicOr(err, 1u);
         }
     } else if (warp == 1) {
-        if (lane == 0) {                                  // MMA issuer
+        if (lane == 0 && rank == 0) {                     // MMA issuer of the pair
             int it = 0, lt = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < g.ntiles && ok; tile += gridDim.x, ++lt) {
+            for (int i = pair; i < g.nitems && ok; i += pairs, ++lt) {
                 const int buf = lt & 1, use = lt >> 1;
                 if (lt >= 2 && !(ok = mbar_wait(&acce[buf], (use - 1) & 1))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc_addr = tmem + (uint32_t)(buf * GBN);
-                const bool ro = g.fused && tile % g.ntn == g.ntn_drive;
-                const uint32_t idesc = ro ? gidesc(g.n_ro) : gidesc(GBN);
+                const uint32_t idesc = gidesc(dense_item(g, i).width);
                 for (int kb = 0; kb < nk; ++kb, ++it) {
                     const int s = it % GSTAGES, round = it / GSTAGES;
                     if (!(ok = mbar_wait(&full[s], round & 1))) break;
@@ -844,18 +890,16 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
                         const uint64_t ad = sdesc(a0) + (uint64_t)(2 * k), bd = sdesc(b0) + (uint64_t)(2 * k);
                         const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u;
                         asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                     "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
                                      :: "r"(acc_addr), "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
                     }
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                                 :: "r"(su32(&empty[s])) : "memory");
+                    snn::tc::mma_commit_pair(&empty[s]);
                 }
                 if (!ok) break;
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             :: "r"(su32(&accf[buf])) : "memory");
+                snn::tc::mma_commit_pair(&accf[buf]);
             }
             // every MMA issued has completed before the tensor memory is freed
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+            asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                          :: "r"(su32(drain)) : "memory");
             if (!mbar_wait(drain, 0)) ok = false;
             if (!ok) atomicOr(err, 1u);
@@ -863,12 +907,15 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
     } else {                                              // epilogue warps
         const int quarter = warp & 3, half = (warp - 2) >> 2;
         int lt = 0;
-        for (int tile = blockIdx.x; tile < g.ntiles; tile += gridDim.x, ++lt) {
-            const int tm = tile / g.ntn, tn = tile % g.ntn;
-            const bool ro = g.fused && tn == g.ntn_drive;
-            const int ncols = ro ? c.n_out : c.N - tn * GBN;   // live columns of the tile
+        for (int i = pair; i < g.nitems; i += pairs, ++lt) {
+            const DenseItem w = dense_item(g, i);
+            const int tm = 2 * w.tmp + rank, tn = w.tn;
+            const bool ro = w.ro;
+            const int j0 = tn * GBN + w.part * w.width;        // the item's first neuron
+            const int ncols = ro ? c.n_out : c.N - j0;         // its live columns (at most `width` of them)
             const int buf = lt & 1, use = lt >> 1;
-            constexpr int CH = GBN / 32 / 2;               // chunks of 32 columns per warp
+            const uint32_t drained = snn::tc::cluster_map(su32(&acce[buf]), 0u);
+            const int steps = ro ? (w.width / 2 + 15) / 16 : w.width / 32;   // 16-column steps per warp
             const int b0 = tm * GBM + quarter * 32;        // the warp's first sample
             const bool got = __all_sync(FULL, mbar_wait(&accf[buf], use & 1) ? 1 : 0) != 0;
             if (!got) {
@@ -878,25 +925,25 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int b = b0 + lane;
             const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * GBN);
-            const bool piped = !ro && (half + 1) * CH * 32 <= ncols && (c.n_in & 1) == 0;
+            const bool piped = !ro && (half + 1) * steps * 16 <= ncols && (c.n_in & 1) == 0;
             if (piped)
-                dense_epilogue_half_pipelined(c, d, tbase + (uint32_t)(half * CH * 32), b, b < c.B,
-                                              tn * GBN + half * CH * 32, cur, nxt, t_local, &acce[buf], g);
+                dense_epilogue_half_pipelined(c, d, tbase + (uint32_t)(half * steps * 16), b, b < c.B,
+                                              j0 + half * steps * 16, steps, cur, nxt, t_local, drained, g);
             // otherwise (a half tile past the layer's end, or the readout tile):
             // 16-column steps, each neuron guarded
             uint32_t word = 0u;
-            for (int q = 0; q < (piped ? 0 : 2 * CH); ++q) {
-                const int col = half * CH * 32 + 16 * q;    // uniform over the warp
+            for (int q = 0; q < (piped ? 0 : steps); ++q) {
+                const int col = (half * steps + q) * 16;    // uniform over the warp
                 uint32_t r[16];
                 if (col < ncols) tmem_ld16(tbase + (uint32_t)col, r);
-                if (q == 2 * CH - 1) {                      // this warp is done with the accumulator
+                if (q == steps - 1) {                      // this warp is done with the accumulator
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(su32(&acce[buf])) : "memory");
+                    if (lane == 0) snn::tc::mbar_arrive_cluster(drained);
                 }
                 if (col >= ncols) continue;
                 if (!ro) {
-                    const int j = tn * GBN + col, nu = min(16, c.N - j);
+                    const int j = j0 + col, nu = min(16, c.N - j);
                     uint32_t w16 = 0u;
                     if (b < c.B) {
                         const size_t q0 = sidx(b, j, c.N);
@@ -936,17 +983,19 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
                 }
             }
             // this warp's share of the next step's input draws: groups of 32 inputs,
-            // alternating between the two column halves
+            // alternating between the column halves of the tile's items
+            const int cut = GBN / w.width;
             if (!ro && g.enc_next)
-                for (int a0 = tn * g.a_per + half * 32; a0 < min(c.n_in, (tn + 1) * g.a_per); a0 += 64)
+                for (int a0 = tn * g.a_per + (w.part * 2 + half) * 32; a0 < min(c.n_in, (tn + 1) * g.a_per); a0 += 64 * cut)
                     dense_encode_group(c, d, b, b < c.B, tt + 1ull, a0);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    snn::tc::cluster_sync();               // no CTA leaves while the other uses its memory
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(2 * GBN) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(2 * GBN) : "memory");
     }
 }
 
@@ -1074,6 +1123,22 @@ __global__ void k_rec_pack(const uint16_t* __restrict__ w_ff, const uint16_t* __
 bool encode_map(CUtensorMap* m, void* base, int rows, int K, int box_rows) {
     static_assert(GBK == snn::tc::KB, "tiles are 64 K-elements wide");
     return snn::tc::encode_bf16_map(m, base, rows, K, box_rows);
+}
+
+cudaError_t launch_dense(const CUtensorMap (&maps)[2], const CUtensorMap& map_w, const RecConsts& c, const RecBufs& d,
+                         int t, const DenseGeom& g, uint32_t* err, unsigned grid, cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(GTHREADS);
+    cfg.dynamicSmemBytes = GSMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_rec_dense, maps[0], maps[1], map_w, c, d, t, g, err);
 }
 
 bool finite_pos(float x) { return std::isfinite(x) && x > 0.0f; }
@@ -1248,8 +1313,7 @@ snn_status snn_rec_create(const snn_rec_spec* spec, snn_rec** out) {
     if (e == cudaSuccess) e = dalloc(&r->step, 2);
     r->geom.ntn_drive = (s.n_hid + GBN - 1) / GBN;
     r->geom.fused = s.n_out <= GBN ? 1 : 0;
-    r->geom.ntn = r->geom.ntn_drive + r->geom.fused;
-    r->geom.n_ro = r->geom.fused ? (s.n_out + 15) / 16 * 16 : 0;
+    r->geom.n_ro = r->geom.fused ? (s.n_out + 31) / 32 * 32 : 0;   // (a pair's products are 32 n wide)
     r->geom.a_per = ((s.n_in + r->geom.ntn_drive - 1) / r->geom.ntn_drive + 31) / 32 * 32;
     r->wt_rows = r->geom.fused ? r->geom.ntn_drive * GBN + s.n_out : s.n_hid;
     if (e == cudaSuccess) e = dalloc(&r->wt, (size_t)r->wt_rows * r->K);
@@ -1279,7 +1343,7 @@ snn_status snn_rec_create(const snn_rec_spec* spec, snn_rec** out) {
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e == cudaSuccess && !encode_map(&r->map_w, r->wt, r->wt_rows, r->K, GBN)) {
+    if (e == cudaSuccess && !encode_map(&r->map_w, r->wt, r->wt_rows, r->K, GWB)) {
         snn_rec_destroy(r);
         return rec_fail(nullptr, SNN_ERR_CUDA, "snn_rec_create: cannot encode the weight tensor map");
     }
@@ -1404,8 +1468,14 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
     REC_TRY(r, cudaGetLastError());
     const size_t enc_warps = (size_t)B * c.Iw, hid_warps = (size_t)B * c.Nw;
     DenseGeom geom = r->geom;
-    geom.ntiles = ((B + GBM - 1) / GBM) * geom.ntn;
-    const unsigned dgrid = (unsigned)std::min(geom.ntiles, r->num_sms);
+    const int pairs = std::max(1, r->num_sms / 2), sample_tiles = (B + 2 * GBM - 1) / (2 * GBM);
+    const int ro_items = geom.fused * sample_tiles;
+    geom.nd = sample_tiles * geom.ntn_drive;
+    const int last = geom.nd % pairs;      // drive tiles of the round that is not full
+    geom.parts = 4 * last + ro_items <= pairs ? 4 : 2 * last + ro_items <= pairs ? 2 : 1;
+    geom.nfull = geom.nd - last;
+    geom.nitems = geom.nfull + geom.parts * last + ro_items;
+    const unsigned dgrid = 2u * (unsigned)std::min(geom.nitems, pairs);   // a pair of CTAs per item
     // the tensor form draws each next step's inputs in the product's epilogue,
     // unless the input raster is recorded
     const bool fuse_enc = dense && !c.rec_input;
@@ -1424,8 +1494,7 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
         geom.keep_sh = !geom.fused || t == T - 1 ? 1 : 0;
         mark(SNN_REC_KERNEL_DRIVE, true);
         if (dense)
-            k_rec_dense<<<dgrid, GTHREADS, GSMEM, st>>>(r->map_s[0], r->map_s[1], r->map_w, c, d, t, geom,
-                                                         r->dev_err);
+            REC_TRY(r, launch_dense(r->map_s, r->map_w, c, d, t, geom, r->dev_err, dgrid, st));
         else
             k_rec_hidden<<<(unsigned)((hid_warps + 7) / 8), 256, 0, st>>>(c, d, t);
         mark(SNN_REC_KERNEL_DRIVE, false);

@@ -72,6 +72,23 @@ __device__ __forceinline__ void tma_2d(void* dst, const CUtensorMap* tm, int c0,
                  "[%0], [%1, {%2, %3}], [%4];"
                  :: "r"(su32(dst)), "l"((uint64_t)tm), "r"(c0), "r"(c1), "r"(su32(bar)) : "memory");
 }
+// The same for a pair of CTAs (cta_group::2): into this CTA's shared memory, the
+// bytes counted on the mbarrier at cluster address `bar`, which may be the peer's.
+__device__ __forceinline__ void tma_2d_pair(void* dst, const CUtensorMap* tm, int c0, int c1, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+                 "[%0], [%1, {%2, %3}], [%4];"
+                 :: "r"(su32(dst)), "l"((uint64_t)tm), "r"(c0), "r"(c1), "r"(bar) : "memory");
+}
+// An arrival on the mbarrier at a cluster address.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" :: "r"(bar) : "memory");
+}
+// The pair's products issued before have finished: an arrival on this mbarrier in
+// both CTAs.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 :: "r"(su32(bar)), "h"((uint16_t)3) : "memory");
+}
 // 16-byte asynchronous copies (through L2 only); cp_async_arrive makes the
 // mbarrier's current phase wait for the calling thread's copies so far (one
 // arrival of its expected count).

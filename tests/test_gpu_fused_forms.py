@@ -4,7 +4,7 @@ against the oracle."""
 import numpy as np
 import pytest
 
-from test_gpu_rec import _built, assert_same, dev, oracle_run, snn, workload  # noqa: F401
+from test_gpu_rec import _built, assert_same, bits, dev, dyadic_workload, oracle_run, snn, workload  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -31,6 +31,29 @@ def test_rec_gather_one_launch(B, NI, N, NO, T):
         net.run(dev(r), dev(s), 3, continue_=True, record=True, record_input=True, form="gather", profile=profile)
         assert_same(net, st, rh, ri)
     net.close()
+
+
+@pytest.mark.parametrize("B,NI,N,NO", [
+    (1, 33, 200, 256),         # one item per part, the widest readout, unpaired operand columns
+    (300, 64, 700, 40),        # tiles in four parts, the last pair of CTAs with 44 samples in one
+    (2200, 40, 700, 10),       # tiles in two parts, ragged in the second
+    (2560, 64, 2000, 10),      # a full round and the rest of the tiles in four parts
+])
+def test_rec_tensor_form_cut_tiles(B, NI, N, NO):
+    """Samples of the first CTA, the second CTA and the last one against oracle
+    runs of that sample alone (dyadic weights)."""
+    T = 12
+    p, r, s, wf, wr, wo = dyadic_workload(B, NI, N, NO, seed=N)
+    net = snn().RecNetwork(p, wf, wr, wo)
+    net.run(dev(r), dev(s), T, record=True, form="tensor")
+    got = {name: net.read(name) for name in ("raster", "v", "i_syn", "v_out", "counts")}
+    net.close()
+    for b in sorted({0, min(B - 1, 131), B - 1}):
+        st, rh, _ = oracle_run(p, r[b:b + 1], s[b:b + 1], wf, wr, wo, T)
+        assert rh.sum() > 0
+        assert np.array_equal(got["raster"][:, b], rh[:, 0]), b
+        for name, ref in (("v", st.v), ("i_syn", st.i_syn), ("v_out", st.v_out), ("counts", st.counts)):
+            assert np.array_equal(bits(got[name][b]), bits(ref[0])), (b, name)
 
 
 @pytest.mark.parametrize("B,NI,N,T,reduce", [
