@@ -114,8 +114,7 @@ constexpr uint16_t BF16_ONE = 0x3F80;
 // neurons with cta_group::2 products: each CTA stages its own 128 samples and half
 // of the neurons' weights, and keeps its samples' accumulator.
 constexpr int GBM = 128, GBN = 256, GBK = 64, GSTAGES = 6;
-constexpr int GWB = GBN / 2;             // weight rows of one TMA copy
-constexpr int GA_BYTES = GBM * GBK * 2, GW_BYTES = GWB * GBK * 2, GSTAGE = GA_BYTES + GBN / 2 * GBK * 2;
+constexpr int GA_BYTES = GBM * GBK * 2, GB_BYTES = GBN / 2 * GBK * 2, GSTAGE = GA_BYTES + GB_BYTES;
 constexpr int GSMEM = GSTAGES * GSTAGE + 1024 + 256;
 constexpr int GEPI_WARPS = 8, GTHREADS = 64 + 32 * GEPI_WARPS;
 constexpr unsigned long long GWAIT_NS = 2000000000ull;   // bounded waits: 2 s, then the error flag
@@ -848,31 +847,40 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
     const CUtensorMap* tmS = cur ? &tmS1 : &tmS0;
     if (warp == 0) {
         if (lane == 0) {                                  // TMA producer
-            int it = 0;
+            // (stage s in its phase ph: a wait for the other parity passes on a fresh
+            // barrier; counters advance rather than being divided out, for a lone
+            // lane's stage has room for few instructions: 147 and 145.5 us a step)
+            const uint32_t full0 = snn::tc::cluster_map(su32(full), 0u);
+            uint32_t s = 0u, ph = 1u;
             bool ok = true;
             for (int i = pair; i < g.nitems && ok; i += pairs) {
                 const DenseItem w = dense_item(g, i);
-                const int tm = 2 * w.tmp + rank, rows = w.width / 2;   // this CTA's half of the weights
-                const int wrow = w.tn * GBN + w.part * w.width + rank * rows, copies = (rows + GWB - 1) / GWB;
-                for (int kb = 0; kb < nk; ++kb, ++it) {
-                    const int s = it % GSTAGES, round = it / GSTAGES;
-                    if (it >= GSTAGES && !(ok = mbar_wait(&empty[s], (round - 1) & 1))) break;
+                const int rows = w.width / 2;              // this CTA's half of the weights
+                const int srow = (2 * w.tmp + rank) * GBM, wrow = w.tn * GBN + w.part * w.width + rank * rows;
+#pragma unroll 1
+                for (int k = 0; k < nk * GBK; k += GBK) {
+                    if (!(ok = mbar_wait(&empty[s], ph))) break;
+                    if (rank == 0) mbar_expect_tx(&full[s], 2 * GSTAGE);
                     uint8_t* st = smem + s * GSTAGE;
-                    const uint32_t f = snn::tc::cluster_map(su32(&full[s]), 0u);
-                    if (rank == 0) mbar_expect_tx(&full[s], 2 * (GA_BYTES + copies * GW_BYTES));
-                    snn::tc::tma_2d_pair(st, tmS, kb * GBK, tm * GBM, f);
-                    for (int q = 0; q < copies; ++q)
-                        snn::tc::tma_2d_pair(st + GA_BYTES + q * GW_BYTES, &tmW, kb * GBK, wrow + q * GWB, f);
+                    const uint32_t f = full0 + 8u * s;
+                    snn::tc::tma_2d_pair(st, tmS, k, srow, f);
+                    snn::tc::tma_2d_pair(st + GA_BYTES, &tmW, k, wrow, f);
+                    if (++s == GSTAGES) s = 0u, ph ^= 1u;
                 }
             }
             // the commits that free the last stages arrive here from the first CTA:
             // this one stays until they have
-            for (int j = max(0, it - GSTAGES); j < it && ok; ++j) ok = mbar_wait(&empty[j % GSTAGES], (j / GSTAGES) & 1);
+            for (int q = 0; q < GSTAGES && ok; ++q) {
+                ok = mbar_wait(&empty[s], ph);
+                if (++s == GSTAGES) s = 0u, ph ^= 1u;
+            }
             if (!ok) atomicOr(err, 1u);
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {                     // MMA issuer of the pair
-            int it = 0, lt = 0;
+            const uint64_t desc0 = sdesc(su32(smem));
+            uint32_t s = 0u, ph = 0u;
+            int lt = 0;
             bool ok = true;
             for (int i = pair; i < g.nitems && ok; i += pairs, ++lt) {
                 const int buf = lt & 1, use = lt >> 1;
@@ -880,20 +888,21 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc_addr = tmem + (uint32_t)(buf * GBN);
                 const uint32_t idesc = gidesc(dense_item(g, i).width);
-                for (int kb = 0; kb < nk; ++kb, ++it) {
-                    const int s = it % GSTAGES, round = it / GSTAGES;
-                    if (!(ok = mbar_wait(&full[s], round & 1))) break;
+#pragma unroll 1
+                for (int kb = 0; kb < nk; ++kb) {
+                    if (!(ok = mbar_wait(&full[s], ph))) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a0 = su32(smem + s * GSTAGE), b0 = a0 + GA_BYTES;
+                    const uint64_t ad = desc0 + s * (uint64_t)(GSTAGE >> 4), bd = ad + (uint64_t)(GA_BYTES >> 4);
 #pragma unroll
                     for (int k = 0; k < GBK / 16; ++k) {      // K = 16 per MMA: +32 bytes in the swizzled row
-                        const uint64_t ad = sdesc(a0) + (uint64_t)(2 * k), bd = sdesc(b0) + (uint64_t)(2 * k);
                         const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u;
                         asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                                      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                                     :: "r"(acc_addr), "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
+                                     :: "r"(acc_addr), "l"(ad + (uint64_t)(2 * k)), "l"(bd + (uint64_t)(2 * k)),
+                                        "r"(idesc), "r"(acc) : "memory");
                     }
                     snn::tc::mma_commit_pair(&empty[s]);
+                    if (++s == GSTAGES) s = 0u, ph ^= 1u;
                 }
                 if (!ok) break;
                 snn::tc::mma_commit_pair(&accf[buf]);
@@ -930,7 +939,10 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
                 dense_epilogue_half_pipelined(c, d, tbase + (uint32_t)(half * steps * 16), b, b < c.B,
                                               j0 + half * steps * 16, steps, cur, nxt, t_local, drained, g);
             // otherwise (a half tile past the layer's end, or the readout tile):
-            // 16-column steps, each neuron guarded
+            // 16-column steps, the state of eight neurons in flight, each store
+            // guarded (with the loads guarded one by one the last tile was the whole
+            // step's end: 64->3000, B = 2500, 105 us a step, 65 so; 300->626, B = 626,
+            // 25.6 and 21.5)
             uint32_t word = 0u;
             for (int q = 0; q < (piped ? 0 : steps); ++q) {
                 const int col = (half * steps + q) * 16;    // uniform over the warp
@@ -947,18 +959,28 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
                     uint32_t w16 = 0u;
                     if (b < c.B) {
                         const size_t q0 = sidx(b, j, c.N);
-#pragma unroll 4
-                        for (int u = 0; u < 16; ++u) {
-                            if (u >= nu) break;
-                            const size_t qq = q0 + 32 * u;
-                            float x = __fmul_rn(c.a_syn, d.i_syn[qq]);
-                            x = __fadd_rn(x, __uint_as_float(r[u]));
-                            d.i_syn[qq] = x;
-                            float y = __fmul_rn(c.a_mem, d.v[qq]);
-                            y = __fadd_rn(y, x);
-                            const bool spk = y >= c.v_thresh;
-                            d.v[qq] = spk ? c.v_reset : y;
-                                            w16 |= (spk ? 1u : 0u) << u;
+#pragma unroll
+                        for (int h = 0; h < 16; h += 8) {
+                            float I[8], V[8];              // all in flight, past the end the last neuron's
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) {
+                                const size_t qq = q0 + 32 * min(h + u, nu - 1);
+                                I[u] = d.i_syn[qq];
+                                V[u] = d.v[qq];
+                            }
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) {
+                                float x = __fmul_rn(c.a_syn, I[u]);
+                                x = __fadd_rn(x, __uint_as_float(r[h + u]));
+                                float y = __fmul_rn(c.a_mem, V[u]);
+                                y = __fadd_rn(y, x);
+                                const bool spk = y >= c.v_thresh;
+                                if (h + u < nu) {
+                                    d.i_syn[q0 + 32 * (h + u)] = x;
+                                    d.v[q0 + 32 * (h + u)] = spk ? c.v_reset : y;
+                                    w16 |= (spk ? 1u : 0u) << (h + u);
+                                }
+                            }
                         }
                         if (c.rec_raster) {
                             uint8_t* rp = d.raster_h + ((size_t)t_local * c.B + b) * c.N + j;
@@ -977,9 +999,12 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
                     // step's operand (the run's first step skips it: the run before
                     // added it)
                     float* vo = d.v_out + (size_t)b * c.n_out;
+                    float y[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) y[u] = vo[min(col + u, c.n_out - 1)];
 #pragma unroll
                     for (int u = 0; u < 16; ++u)
-                        if (col + u < c.n_out) vo[col + u] = __fadd_rn(vo[col + u], __uint_as_float(r[u]));
+                        if (col + u < c.n_out) vo[col + u] = __fadd_rn(y[u], __uint_as_float(r[u]));
                 }
             }
             // this warp's share of the next step's input draws: groups of 32 inputs,
@@ -1343,7 +1368,7 @@ snn_status snn_rec_create(const snn_rec_spec* spec, snn_rec** out) {
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e == cudaSuccess && !encode_map(&r->map_w, r->wt, r->wt_rows, r->K, GWB)) {
+    if (e == cudaSuccess && !encode_map(&r->map_w, r->wt, r->wt_rows, r->K, GBN / 2)) {
         snn_rec_destroy(r);
         return rec_fail(nullptr, SNN_ERR_CUDA, "snn_rec_create: cannot encode the weight tensor map");
     }
