@@ -846,7 +846,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
     const int cur = (int)(tt & 1ull), nxt = cur ^ 1;
     const CUtensorMap* tmS = cur ? &tmS1 : &tmS0;
     if (warp == 0) {
-        if (lane == 0) {                                  // TMA producer
+        if (snn::tc::elect_one()) {                       // TMA producer
             // (stage s in its phase ph: a wait for the other parity passes on a fresh
             // barrier; counters advance rather than being divided out, for a lone
             // lane's stage has room for few instructions: 147 and 145.5 us a step)
@@ -877,7 +877,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
             if (!ok) atomicOr(err, 1u);
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {                     // MMA issuer of the pair
+        if (rank == 0 && snn::tc::elect_one()) {          // MMA issuer of the pair
             const uint64_t desc0 = sdesc(su32(smem));
             uint32_t s = 0u, ph = 0u;
             int lt = 0;

@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_current(const __grid_consta
     const unsigned long long tt = d.step[0] + (unsigned long long)t_local;
     const int p3 = (int)(tt % 3ull);
     if (warp == 0) {
-        if (lane == 0) {                                      // TMA producer
+        if (elect_one()) {                                    // TMA producer
             int it = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_current(const __grid_consta
             drain_loads(full, it, CUR_STAGES);
         }
     } else if (warp == 1) {
-        if (lane == 0) {                                      // MMA issuer
+        if (elect_one()) {                                    // MMA issuer
             const uint32_t idesc = idesc_bf16(t.TB);
             int it = 0, lt = 0;
             bool ok = true;
@@ -678,14 +678,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
     const int nch = t.TNI / 16;
     const int ch0 = ks + t.KS * half, chs = 2 * t.KS;
     WChunk<MASTER> wc;
-    if (warp == 0) {                                          // TMA producer (lane 0)
+    if (warp == 0) {                                          // TMA producer (one lane)
         SlotWalk sw;
         bool ok = true;
         uint32_t used = 0u;                                   // slots ever filled
         for (int tile = first; tile < end; tile += step) {
             const int tm = tile_m(tile), tn = tile_n(tile);
             read_marks(tm);
-            if (lane != 0) continue;
+            if (!elect_one()) continue;
             for (int it = 0; it < nk && ok; ++it) {
                 const bool post = has_post(it);
                 const int s = sw.next(post);
@@ -711,20 +711,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
                 sw.take(s, post);
             }
         }
-        if (lane == 0) {
+        if (elect_one()) {
             if (!ok) atomicOr(d.err, ERR_TENSOR);
             // every copy issued has landed before the CTA may leave
             for (int s = 0; s < DW_SLOTS; ++s)
                 if ((used >> s) & 1u) mbar_wait(&full[s], sw.last_fill(s), WAIT_NS);
         }
-    } else if (warp == 1) {                                   // MMA issuer (lane 0)
+    } else if (warp == 1) {                                   // MMA issuer (one lane)
         const uint32_t idesc = idesc_bf16(t.TNI);
         SlotWalk sw;
         bool ok = true;
         int lt = 0;
         for (int tile = first; tile < end; tile += step, ++lt) {
             read_marks(tile_m(tile));
-            if (lane != 0 || !ok) continue;
+            if (!elect_one() || !ok) continue;
             const int buf = lt & 1;
             if (lt >= 2 && !(ok = mbar_wait(&acce[buf], ((lt >> 1) - 1) & 1, WAIT_NS))) continue;
             fence_after();
@@ -757,7 +757,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_t_dw(const __grid_constant__ 
             }
             if (ok) mma_commit(&accf[buf]);
         }
-        if (lane == 0) {
+        if (elect_one()) {
             if (!ok) atomicOr(d.err, ERR_TENSOR);
             mma_commit(drain);
             if (!mbar_wait(drain, 0, WAIT_NS)) atomicOr(d.err, ERR_TENSOR);
