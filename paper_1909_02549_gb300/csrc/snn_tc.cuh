@@ -161,6 +161,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
                  : "r"(taddr) : "memory");
 }
 
+// In a launch with programmatic serialization: waits until the launch before has
+// finished and its writes are visible, then lets the launch after begin (its blocks
+// take their places as this one's leave, and wait in turn).
+__device__ __forceinline__ void after_previous_launch() {
+    asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Thread-block clusters: every thread of every CTA of the cluster arrives and
 // waits (release / acquire: shared-memory writes before the barrier are seen
 // by other CTAs' reads after it).  Without .aligned, so a warp need not be

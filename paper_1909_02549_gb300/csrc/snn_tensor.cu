@@ -344,7 +344,9 @@ __device__ __forceinline__ void drain_loads(uint64_t* full, int issued, int S) {
 // the operands' way from L2.  784->6400, B = 1024, a step of 250: with a launch of
 // 400 CTAs, product (8 to 14 us) and epilogue one after the other, 55.3 ms a run;
 // 49.0 with the epilogue's chains side by side; 44.5 with this overlap here and in
-// k_t_dw (BF16 at B = 256: 21.1, 19.7 and 16.4 ms).
+// k_t_dw (BF16 at B = 256: 21.1, 19.7 and 16.4 ms); 37.8 and 14.8 since one elected
+// lane issues the products.  12 epilogue warps: 37.9 and 15.1; the state loaded in
+// eighths of 8 samples, three in flight: 40.5 and 15.4.
 __global__ void __launch_bounds__(TC_THREADS, 1) k_t_current(const __grid_constant__ CUtensorMap mW,
                                                              const __grid_constant__ CUtensorMap mS,
                                                              Consts c, Bufs d, TBufs t, int t_local) {
