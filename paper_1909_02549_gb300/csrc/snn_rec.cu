@@ -813,6 +813,7 @@ __device__ __forceinline__ void dense_epilogue_half_pipelined(const RecConsts& c
 __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant__ CUtensorMap tmS0,
                                                            const __grid_constant__ CUtensorMap tmS1,
                                                            const __grid_constant__ CUtensorMap tmW,
+                                                           const __grid_constant__ CUtensorMap tmWc,
                                                            RecConsts c, RecBufs d, int t_local, DenseGeom g,
                                                            uint32_t* err) {
     extern __shared__ uint8_t smem_raw[];
@@ -857,15 +858,20 @@ __global__ void __launch_bounds__(GTHREADS, 1) k_rec_dense(const __grid_constant
             for (int i = pair; i < g.nitems && ok; i += pairs) {
                 const DenseItem w = dense_item(g, i);
                 const int rows = w.width / 2;              // this CTA's half of the weights
+                // (a narrow item copies half of the rows: 1024->4096, B = 64 27.0 us a
+                // step with all 128, 24.8 with 64, no less with 32; B = 256 28.5 and 26.6)
+                const bool cut = rows <= GBN / 4;
+                const CUtensorMap* tw = cut ? &tmWc : &tmW;
+                const uint32_t bytes = 2u * (cut ? GSTAGE - GB_BYTES / 2 : GSTAGE);
                 const int srow = (2 * w.tmp + rank) * GBM, wrow = w.tn * GBN + w.part * w.width + rank * rows;
 #pragma unroll 1
                 for (int k = 0; k < nk * GBK; k += GBK) {
                     if (!(ok = mbar_wait(&empty[s], ph))) break;
-                    if (rank == 0) mbar_expect_tx(&full[s], 2 * GSTAGE);
+                    if (rank == 0) mbar_expect_tx(&full[s], bytes);
                     uint8_t* st = smem + s * GSTAGE;
                     const uint32_t f = full0 + 8u * s;
                     snn::tc::tma_2d_pair(st, tmS, k, srow, f);
-                    snn::tc::tma_2d_pair(st + GA_BYTES, &tmW, k, wrow, f);
+                    snn::tc::tma_2d_pair(st + GA_BYTES, tw, k, wrow, f);
                     if (++s == GSTAGES) s = 0u, ph ^= 1u;
                 }
             }
@@ -1151,8 +1157,9 @@ bool encode_map(CUtensorMap* m, void* base, int rows, int K, int box_rows) {
     return snn::tc::encode_bf16_map(m, base, rows, K, box_rows);
 }
 
-cudaError_t launch_dense(const CUtensorMap (&maps)[2], const CUtensorMap& map_w, const RecConsts& c, const RecBufs& d,
-                         int t, const DenseGeom& g, uint32_t* err, unsigned grid, cudaStream_t st) {
+cudaError_t launch_dense(const CUtensorMap (&maps)[2], const CUtensorMap& map_w, const CUtensorMap& map_wc,
+                         const RecConsts& c, const RecBufs& d, int t, const DenseGeom& g, uint32_t* err,
+                         unsigned grid, cudaStream_t st) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(GTHREADS);
@@ -1171,7 +1178,7 @@ cudaError_t launch_dense(const CUtensorMap (&maps)[2], const CUtensorMap& map_w,
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_rec_dense, maps[0], maps[1], map_w, c, d, t, g, err);
+    return cudaLaunchKernelEx(&cfg, k_rec_dense, maps[0], maps[1], map_w, map_wc, c, d, t, g, err);
 }
 
 bool finite_pos(float x) { return std::isfinite(x) && x > 0.0f; }
@@ -1186,9 +1193,9 @@ struct snn_rec {
     uint16_t* w_out = nullptr;
     uint16_t* wt = nullptr;            // [wt_rows][K] stacked transposed weights of the dense form
     int K = 0;
-    DenseGeom geom{};                  // per batch: ntiles depends on B
+    DenseGeom geom{};                  // per batch: the items depend on B
     int wt_rows = 0;
-    CUtensorMap map_w{}, map_s[2]{};
+    CUtensorMap map_w[2]{}, map_s[2]{};
     uint32_t* dev_err = nullptr;       // [2]: a dense step's pipeline wait timed out; bad spike bytes
     unsigned long long* act_dev = nullptr;   // hidden spikes of the last run
     unsigned long long* act_host = nullptr;  // pinned copy
@@ -1376,7 +1383,8 @@ snn_status snn_rec_create(const snn_rec_spec* spec, snn_rec** out) {
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e == cudaSuccess && !encode_map(&r->map_w, r->wt, r->wt_rows, r->K, GBN / 2)) {
+    if (e == cudaSuccess && (!encode_map(&r->map_w[0], r->wt, r->wt_rows, r->K, GBN / 2) ||
+                             !encode_map(&r->map_w[1], r->wt, r->wt_rows, r->K, GBN / 4))) {
         snn_rec_destroy(r);
         return rec_fail(nullptr, SNN_ERR_CUDA, "snn_rec_create: cannot encode the weight tensor map");
     }
@@ -1527,7 +1535,7 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
         geom.keep_sh = !geom.fused || t == T - 1 ? 1 : 0;
         mark(SNN_REC_KERNEL_DRIVE, true);
         if (dense)
-            REC_TRY(r, launch_dense(r->map_s, r->map_w, c, d, t, geom, r->dev_err, dgrid, st));
+            REC_TRY(r, launch_dense(r->map_s, r->map_w[0], r->map_w[1], c, d, t, geom, r->dev_err, dgrid, st));
         else
             k_rec_hidden<<<(unsigned)((hid_warps + 7) / 8), 256, 0, st>>>(c, d, t);
         mark(SNN_REC_KERNEL_DRIVE, false);
