@@ -27,12 +27,14 @@
 // The arithmetic is the per-step kernels' (same intrinsics, same order), so the
 // three run modes give bit-identical results.
 //
-// Loops are not unrolled unless that is written out or they are the separate
-// neuron passes' and the quiet-column pass's: the step's code does not fit the
-// instruction cache (92 % of its requests hit at 784->6400, 74 % at 784->100 with
-// the post-triggered rule), and unrolled it was half as large again.  784->6400, B =
-// 256: 7.05 ms a presentation unrolled, 6.82 so; 784->400, B = 1024: 8.58, 8.53;
-// the separate passes' loops are faster unrolled (784->100, B = 64: 3.07 and 3.52).
+// Loops are not unrolled (a pragma each) unless that is written out or they are the
+// separate neuron passes', the quiet-column pass's, the encode's or the first STDP
+// pass's around its calls: the step's code does not fit the instruction cache (92 % of
+// its requests hit at 784->6400, 74 % at 784->100 with the post-triggered rule), and
+// unrolled it was half as large again.  Per step, all unrolled / all rolled / so:
+// 784->6400, B = 256 30.6 / 29.6 / 29.6 us; 784->400, B = 1024 33.1 / 32.7 / 32.4;
+// 784->100, B = 64, rule, max 13.3 / 11.8 / 11.6; 100->1000, B = 1024 60.0 / 60.8 /
+// 60.0; 100->10000, B = 256 64.8 / 65.7 / 64.9.
 #include <cfloat>
 #include <mutex>
 
@@ -241,7 +243,6 @@ __device__ __forceinline__ void encode_words(const Consts& c, const Bufs& d, con
     const int units = nmy * c.Iw;
     // a warp takes two (sample, 32-input word) units per pass: the loads of
     // both are issued before either draw is used
-#pragma unroll 1
     for (int u0 = warp; u0 < units; u0 += 2 * (PT / 32)) {
         int rr[2], iws[2], bs[2];
         bool on[2];
@@ -297,24 +298,20 @@ __device__ __forceinline__ void encode_lists(const Consts& c, const Bufs& d, con
     const int cur = (int)(tt & 1ull);
     const uint32_t* wbuf = (const uint32_t*)(sm + L.o_wbuf);
     const int nmy = cta < c.B ? (c.B - cta + L.G - 1) / L.G : 0;
-#pragma unroll 1
     for (int r = warp; r < nmy; r += PT / 32) {       // one warp per sample
         const int b = cta + L.G * r;
         uint16_t* out = d.act_idx + ((size_t)cur * c.B + b) * c.n_in;
         uint32_t running = 0;
-#pragma unroll 1
         for (int w0 = 0; w0 < c.Iw; w0 += 32) {
             const int w = w0 + lane;
             uint32_t word = w < c.Iw ? wbuf[r * c.Iw + w] : 0u;
             const uint32_t n = __popc(word);
             uint32_t incl = n;
-#pragma unroll 1
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y = __shfl_up_sync(FULL, incl, o);
                 if (lane >= o) incl += y;
             }
             uint32_t off = running + incl - n;
-#pragma unroll 1
             while (word) {
                 const int bit = __ffs(word) - 1;
                 word &= word - 1;
@@ -340,7 +337,6 @@ __device__ __forceinline__ void encode_phase(const Consts& c, const Bufs& d, con
 __device__ __forceinline__ void list_post_columns(const uint32_t* Qm, int nc, int Bw, uint32_t* nzQ,
                                                   uint32_t* nzQw, int* pcol, int* npc_out, int lane) {
     int npc = 0;
-#pragma unroll 1
     for (int jl0 = 0; jl0 < nc; jl0 += 32) {
         const int jl = jl0 + lane;
         int n = 0;
@@ -848,7 +844,9 @@ __device__ __noinline__ void update_post_column_groups(
         if (c.dep_on && lists) {   // every input-spike sample (e is 0 where j has not fired)
             int e0, e1;
             row_span(offs, i, e0, e1);
-#pragma unroll 1
+            // (us a step at 100->1000, B = 1024 and 784->6400, B = 256: rolled 60.6, 29.6;
+            // by three 60.0, 29.7; by four 60.2, 29.9)
+#pragma unroll 3
             for (int e = e0; e < e1; ++e) {
                 const float* er = Es + (int)lst[e] * nst;
 #pragma unroll
@@ -1650,7 +1648,6 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                              // read back, each row's nonzero words from the 8 lanes of its row
                 cp_async_wait_all();
                 const int nch = NI * 8;
-#pragma unroll 1
                 for (int k0 = tid - (tid & 31); k0 < nch; k0 += PT) {
                     const int k = k0 + (tid & 31);
                     uint32_t nz = 0u;
@@ -1667,12 +1664,10 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             } else if (L.masks) {   // the step's masks, padded rows, and each row's nonzero words:
                              // a thread per row, its words in 16-byte loads issued together
                 const uint32_t* src = d.preT + (size_t)(tt % PRET_SLOTS) * NI * Bw;
-#pragma unroll 1
                 for (int i = tid; i < NI; i += PT) {
                     const uint32_t* row = src + (size_t)i * Bw;
                     uint32_t nz = 0u;
                     if ((Bw & 3) == 0) {
-#pragma unroll 1
                         for (int w0 = 0; w0 < Bw; w0 += 16) {
                             uint4 q[4];
 #pragma unroll
@@ -1692,7 +1687,6 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                             }
                         }
                     } else {
-#pragma unroll 1
                         for (int w = 0; w < Bw; ++w) {
                             const uint32_t m = __ldcg(&row[w]);
                             preS[i * PS + w] = m;
@@ -1703,7 +1697,6 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                 }
             } else if (c.reduce == SNN_REDUCE_MAX || !lists) {   // the step's masks, padded rows
                 const uint32_t* src = d.preT + (size_t)(tt % PRET_SLOTS) * NI * Bw;
-#pragma unroll 1
                 for (int k = tid; k < NI * Bw; k += PT) preS[(k / Bw) * PS + (k % Bw)] = __ldcg(&src[k]);
             }
             if (!early) __syncthreads();
@@ -1713,7 +1706,6 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             //     rule has none; it clips every weight, and a column scaled to its
             //     weight sum may have left the bounds)
             if (c.rule == SNN_RULE_POST_NORM) {
-#pragma unroll 1
                 for (int k = tid; k < NI * nc; k += PT) {
                     const int i = k / nc, jl = k % nc;
                     if (nzQ[jl] == 0u) Ws[i * nst + jl] = fminf(fmaxf(Ws[i * nst + jl], c.w_min), c.w_max);
@@ -1754,7 +1746,6 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                 // post-spiking samples, the same for every lane, XC at a time with
                 // their x_pre loads issued together; depression over the lane's own
                 // (input spike and neuron-has-fired) samples.
-#pragma unroll 1
                 for (int u = warp; u < (grouped ? 0 : ntask); u += NW) {
                     const int jl = pcol[u / nch];
                     const int i = (u % nch) * 32 + lane;
@@ -1765,13 +1756,11 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                     int nev = 0;
                     int w = 0;
                     uint32_t qb = Qm[jl];
-#pragma unroll 1
                     for (;;) {
                         int bs[XC];
                         int n = 0;
 #pragma unroll
                         for (int z = 0; z < XC; ++z) {
-#pragma unroll 1
                             while (qb == 0u && w + 1 < Bw) qb = Qm[++w * nc + jl];
                             bs[z] = -1;
                             if (qb) {
@@ -1808,7 +1797,6 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                     if (lists && dep_on) {   // every input-spike sample (e is 0 where j has not fired)
                         int e0, e1;
                         row_span(offs, i, e0, e1);
-#pragma unroll 1
                         for (int e = e0; e < e1; ++e) {
                             const int b = lst[e];
                             if (is_max && ((Qm[(b >> 5) * nc + jl] >> (b & 31)) & 1u)) continue;
@@ -1818,7 +1806,6 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                         }
                     }
                     uint32_t words = lists ? 0u : (Bw <= 32 ? nzP[i] : 0xFFFFFFFFu);
-#pragma unroll 1
                     for (int ww = 0; ww < (lists || !dep_on ? 0 : Bw); ++ww) {
                         if (Bw <= 32) {
                             if (!words) break;
@@ -1827,7 +1814,6 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
                         }
                         uint32_t m = Pi[ww] & Sm[ww * nc + jl];
                         if (is_max) m &= ~Qm[ww * nc + jl];     // post samples were handled above
-#pragma unroll 1
                         while (m) {
                             const int bit = __ffs(m) - 1;
                             m &= m - 1;
