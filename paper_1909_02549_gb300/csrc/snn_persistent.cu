@@ -31,10 +31,12 @@
 // separate neuron passes', the quiet-column pass's, the encode's or the first STDP
 // pass's around its calls: the step's code does not fit the instruction cache (92 % of
 // its requests hit at 784->6400, 74 % at 784->100 with the post-triggered rule), and
-// unrolled it was half as large again.  Per step, all unrolled / all rolled / so:
-// 784->6400, B = 256 30.6 / 29.6 / 29.6 us; 784->400, B = 1024 33.1 / 32.7 / 32.4;
-// 784->100, B = 64, rule, max 13.3 / 11.8 / 11.6; 100->1000, B = 1024 60.0 / 60.8 /
-// 60.0; 100->10000, B = 256 64.8 / 65.7 / 64.9.
+// unrolled it was half as large again.  The step's start is unrolled in the narrow
+// instantiation only.  Per step, all unrolled / so: 784->6400, B = 256 30.5 / 29.7 us;
+// 784->400, B = 1024 33.1 / 32.8; 784->100, B = 64, rule, max 13.3 / 11.7; 225->290, B =
+// 644 17.8 / 17.4; 1023->426, B = 608 35.5 / 35.7; 784->321, B = 115, FP8, max 14.4 /
+// 14.2; 100->1000, B = 1024 59.8 / 60.0; 100->10000, B = 256 64.8 / 64.9.  (All rolled:
+// 29.6, 32.7, 11.8, 18.2, 35.9, 14.5, 60.8, 65.7.)
 #include <cfloat>
 #include <mutex>
 
@@ -1468,13 +1470,13 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             thj[jl] = __fadd_rn(c.e_thresh, __double2float_rn(thS[jl]));
         }
         if (cta == 0)   // accumulator of the next step (its last reader was step tt-1)
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
             for (int b = tid; b < B; b += PT) d.cnt[(size_t)((p3 + 1) % 3) * B + b] = 0u;
         {   // input-major masks of step tt+2, slot of step tt-2: every CTA has run
             // that step's STDP before signalling its encode of step tt
             const size_t n_pre = (size_t)NI * Bw;
             uint32_t* z = d.preT + (size_t)((tt + 2ull) % PRET_SLOTS) * n_pre;
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
             for (size_t k = (size_t)cta * PT + tid; k < n_pre; k += (size_t)G * PT) z[k] = 0u;
         }
         // the previous step's inhibitory counts and this step's active-input counts
@@ -1482,7 +1484,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             cntS[tid] = cn0;
             actN[tid] = an0;
         }
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
         for (int b = tid + PT; b < B; b += PT) {
             cntS[b] = __ldcg(&cnt_src[b]);
             actN[b] = __ldcg(&actn_src[b]);
@@ -1490,7 +1492,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
         // first entries of every sample's active-input list (in bounds: caps <= n_in)
         if (acts_vec) {
             if (tid < acts_n) ((uint4*)actS)[tid] = av0;
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
             for (int k0 = tid + PT; k0 < acts_n; k0 += 2 * PT) {
                 uint4 v4[2];
 #pragma unroll
@@ -1506,7 +1508,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             }
         } else {
             const int n = B * caps;
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
             for (int k = tid; k < n; k += PT)
                 actS[(k / caps) * CAPS + (k % caps)] = __ldcg(&acts_src[(size_t)(k / caps) * NI + (k % caps)]);
         }
@@ -1525,7 +1527,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
             const int nwr = NI < PT ? (NI + 31) / 32 : NW;   // warps with rows
             const int capw = L.lcap / nwr, reg0 = wp * capw;
             int run = 0;                                     // the warp's entries so far
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
             for (int r0 = 0; r0 < NI; r0 += PT) {
                 const int i = r0 + tid;
                 uint32_t wr[8];                              // the row's words
@@ -1592,12 +1594,12 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
         if (t + 1 < T) encode_words(c, d, L, sm, tt + 1, t + 1);
         if (c.wprec == SNN_W_FP8E4M3) {   // column scales of this step's weights
             const int warp = tid >> 5, lane = tid & 31;
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
             for (int jl = warp; jl < nc; jl += NW) {
                 float m = 0.0f;
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
                 for (int i = lane; i < NI; i += 32) m = fmaxf(m, fabsf(Ws[i * nst + jl]));
-#pragma unroll 1
+#pragma unroll
                 for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
                 if (lane == 0) {
                     const float sc = e4m3_scale_of(m);
