@@ -670,7 +670,7 @@ __device__ __forceinline__ void dense_encode_group(const RecConsts& c, const Rec
 __device__ __forceinline__ void keep_word(const RecConsts& c, const RecBufs& d, const DenseGeom& g, int b, int jw,
                                           int cur, uint32_t word) {
     const size_t bp = (size_t)((c.B + 31) >> 5);
-    d.hist[(((size_t)g.slot * bp + (b >> 5)) * c.Nw + jw) * 32 + (b & 31)] = word;
+    if (d.hist) d.hist[(((size_t)g.slot * bp + (b >> 5)) * c.Nw + jw) * 32 + (b & 31)] = word;
     if (g.keep_sh) d.sh[((size_t)cur * c.B + b) * c.Nw + jw] = word;
 }
 
@@ -679,8 +679,9 @@ __device__ __forceinline__ void keep_word(const RecConsts& c, const RecBufs& d, 
 // counts are read and written once for n steps.  In the product's epilogue they
 // were a third of its state bytes, every step, and the registers of a third
 // pipeline slot: 1024->4096, B = 4096, T = 500 took 85.3 ms, 78.9 with them here
-// (171 and 157 us a step).
-__global__ void __launch_bounds__(256) k_rec_fold(RecConsts c, RecBufs d, int n) {
+// (171 and 157 us a step).  Without hist (see snn_rec_run) the counts take each
+// step's words from sh.
+__global__ void __launch_bounds__(256) k_rec_fold(RecConsts c, RecBufs d, int t_local, int n) {
     const int lane = threadIdx.x & 31;
     const size_t gw = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const size_t bp = (size_t)((c.B + 31) >> 5);
@@ -690,7 +691,9 @@ __global__ void __launch_bounds__(256) k_rec_fold(RecConsts c, RecBufs d, int n)
     uint32_t k0 = 0u, k1 = 0u, k2 = 0u, k3 = 0u, k4 = 0u;
 #pragma unroll 8
     for (int s = 0; s < n; ++s) {
-        uint32_t x = d.hist[((size_t)s * bp * c.Nw + gw) * 32 + lane], t;
+        uint32_t x, t;
+        if (d.hist) x = d.hist[((size_t)s * bp * c.Nw + gw) * 32 + lane];
+        else x = d.sh[((size_t)((d.step[0] + (unsigned long long)t_local) & 1ull) * c.B + b) * c.Nw + jw];   // n = 1
         t = k0 & x; k0 ^= x; x = t;
         t = k1 & x; k1 ^= x; x = t;
         t = k2 & x; k2 ^= x; x = t;
@@ -1480,9 +1483,17 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
         form = (r->activity >= 0.0 && r->activity < cut) ? SNN_REC_GATHER : SNN_REC_TENSOR;
     }
     const int dense = form == SNN_REC_TENSOR ? 1 : 0;
+    // the spike words' ring of the tensor form, with its first run of this batch size;
+    // where it cannot be had (no memory left, or a capture that forbids allocation)
+    // the counts are updated every step instead
     if (dense && !r->d.hist) {
-        if (r->last) REC_TRY(r, cudaStreamSynchronize(r->last));
-        REC_TRY(r, dalloc(&r->d.hist, (size_t)HIST * state_elems(B, c.Nw)));
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        REC_TRY(r, cudaStreamIsCapturing(st, &capturing));
+        if (capturing == cudaStreamCaptureStatusNone &&
+            dalloc(&r->d.hist, (size_t)HIST * state_elems(B, c.Nw)) != cudaSuccess) {
+            r->d.hist = nullptr;
+            (void)cudaGetLastError();
+        }
     }
     const bool profile = (flags & SNN_PROFILE) != 0;
     r->last_profiled = false;
@@ -1531,17 +1542,17 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
             mark(SNN_REC_KERNEL_ENCODE, false);
         }
         geom.enc_next = fuse_enc && t + 1 < T ? 1 : 0;
-        geom.slot = t % HIST;
-        geom.keep_sh = !geom.fused || t == T - 1 ? 1 : 0;
+        geom.slot = d.hist ? t % HIST : 0;
+        geom.keep_sh = !d.hist || !geom.fused || t == T - 1 ? 1 : 0;
         mark(SNN_REC_KERNEL_DRIVE, true);
         if (dense)
             REC_TRY(r, launch_dense(r->map_s, r->map_w[0], r->map_w[1], c, d, t, geom, r->dev_err, dgrid, st));
         else
             k_rec_hidden<<<(unsigned)((hid_warps + 7) / 8), 256, 0, st>>>(c, d, t);
         mark(SNN_REC_KERNEL_DRIVE, false);
-        if (dense && (geom.slot == HIST - 1 || t == T - 1)) {
+        if (dense && (!d.hist || geom.slot == HIST - 1 || t == T - 1)) {
             const size_t warps = (size_t)((B + 31) / 32) * c.Nw;
-            k_rec_fold<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(c, d, geom.slot + 1);
+            k_rec_fold<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(c, d, t, geom.slot + 1);
         }
         // the tensor form's product adds each step's readout one step later;
         // the run's last step is read out here

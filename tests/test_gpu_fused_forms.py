@@ -56,6 +56,31 @@ def test_rec_tensor_form_cut_tiles(B, NI, N, NO):
             assert np.array_equal(bits(got[name][b]), bits(ref[0])), (b, name)
 
 
+def test_rec_tensor_form_counts_without_their_ring():
+    """A tensor run recorded by a capture, the first of its batch size, may not
+    allocate: the counts then take each step's spikes."""
+    B, NI, N, NO, T = 130, 64, 300, 10, 40
+    p, r, s, wf, wr, wo = dyadic_workload(B, NI, N, NO, seed=3)
+    st, rh, _ = oracle_run(p, r, s, wf, wr, wo, T)
+    assert rh.sum() > 0
+    net = snn().RecNetwork(p, wf, wr, wo)
+    R, S = dev(r), dev(s)
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        net.run(R, S, 3, form="gather")
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="relaxed"):
+        net.run(R, S, T, form="tensor")
+    for _ in range(2):
+        graph.replay()
+        torch.cuda.synchronize()
+        for name, ref in (("v", st.v), ("i_syn", st.i_syn), ("v_out", st.v_out), ("counts", st.counts)):
+            assert np.array_equal(bits(net.read(name)), bits(ref)), name
+    net.close()
+
+
 @pytest.mark.parametrize("B,NI,N,T,reduce", [
     (3, 7, 1, 60, "mean"),         # one column, fewer inputs than a list's load
     (37, 100, 6007, 8, "sum"),     # 16 columns a block, rows that are not 16-byte aligned, a short last tile
