@@ -355,6 +355,9 @@ __global__ void __launch_bounds__(32 * (GNW_MAX + GE), 1) k_rec_gather(RecConsts
     for (int a = tid; a < c.n_in; a += blockDim.x) thr[a] = d.thr[sidx(b, a, c.n_in)];
     for (int w = tid; w < c.Nw; w += blockDim.x)           // hidden spikes of the step before the first
         words[c.Iw + w] = d.sh[((size_t)((base + 1ull) & 1ull) * c.B + b) * c.Nw + w];
+    // input words of the other buffer: with T = 1 no step draws them, and the closing
+    // list reads them (bits past n_in would lengthen it beyond its room)
+    for (int w = tid; w < c.Iw; w += blockDim.x) words[IN + w] = 0u;
     float vout = 0.0f;                                     // CTA 0, readout warp: output `lane`
     const bool streams = !is_neuron && warp < g.nw + GSW, reads_out = rank == 0 && warp == g.nw + GSW;
     if (reads_out && lane < c.n_out) vout = d.v_out[(size_t)b * c.n_out + lane];

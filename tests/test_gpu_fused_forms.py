@@ -159,3 +159,23 @@ def test_small_batch_cluster(B, NI, N, T, reduce, wprec):
         tp.assert_parity(g, st, rec)
         assert k > 0 or rec.raster_e.sum() > 0
     net.close()
+
+
+@pytest.mark.parametrize("B,NI,N,NO", [
+    (3, 33, 31, 10),           # 31 bits of the last input word past the inputs
+    (2, 1, 700, 3),            # one input; clusters
+    (1, 1025, 64, 40),         # 33 input words, more outputs than lanes
+])
+def test_rec_gather_runs_of_one_step(B, NI, N, NO):
+    """Runs of a single step: the closing list, for the readout of that step, holds
+    its hidden spikes alone (no input words are drawn for a step after it)."""
+    p, r, s, wf, wr, wo = workload(B, NI, N, NO, seed=NI, ff_gain=64.0)
+    r = np.full_like(r, 600.0)
+    net, st, fired = snn().RecNetwork(p, wf, wr, wo), None, 0
+    for t in range(12):
+        st, rh, ri = oracle_run(p, r, s, wf, wr, wo, 1, st=st, episodic=t == 0)
+        net.run(dev(r), dev(s), 1, continue_=t > 0, record=True, record_input=True, form="gather")
+        assert_same(net, st, rh, ri)
+        fired += int(rh.sum())
+    assert fired > 0
+    net.close()
