@@ -542,7 +542,7 @@ cudaError_t launch_cols_step(const Consts& c, const Bufs& d, int t_local, int T,
     auto kern = c.reduce == SNN_REDUCE_SUM    ? (v4 ? k_cols<SNN_REDUCE_SUM, true> : k_cols<SNN_REDUCE_SUM, false>)
                 : c.reduce == SNN_REDUCE_MEAN ? (v4 ? k_cols<SNN_REDUCE_MEAN, true> : k_cols<SNN_REDUCE_MEAN, false>)
                                               : (v4 ? k_cols<SNN_REDUCE_MAX, true> : k_cols<SNN_REDUCE_MAX, false>);
-    if (t_local == 0 && g.smem > 48 * 1024) {
+    if (t_local == 0) {   // (the default limit, 48 KB, counts the kernel's static shared memory too)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
         if (e != cudaSuccess) return e;
     }

@@ -59,7 +59,7 @@ cudaError_t launch_infer(const Consts& c, const Bufs& d, int T, cudaStream_t s, 
     cudaError_t e;
     if (c.wprec == SNN_W_FP8E4M3 && (e = launch_colscale(c, d, s)) != cudaSuccess) return e;
     auto kern = npt == 1 ? k_infer<1> : npt == 2 ? k_infer<2> : npt == 4 ? k_infer<4> : k_infer<8>;
-    if (smem > 48 * 1024) {
+    if (smem > SAMPLE_SMEM_DEFAULT) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
     }

@@ -34,6 +34,10 @@ struct SampleIO {
     size_t rs_n, rs_i;         // words between steps of the rasters
 };
 
+// Dynamic shared memory that a kernel of run_sample may use without an opt-in: the
+// default 48 KB less the static arrays of run_sample (144 bytes), which count too.
+constexpr size_t SAMPLE_SMEM_DEFAULT = 48 * 1024 - 256;
+
 struct SampleSmem {
     size_t o_idx, o_act, o_words, o_x, o_rec, bytes;   // after the live inputs' thresholds
 };

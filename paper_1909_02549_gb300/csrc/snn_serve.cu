@@ -524,7 +524,7 @@ snn_status snn_serve_step(snn_server* s, int k, void* stream_, int* steps_run) {
     if (nl > 0) {
         const int npt = NI <= 65535 ? snn::sample_npt(N) : 0;
         const size_t need = snn::sample_smem(NI, s->c.Iw, false, false).bytes;
-        if (npt == 0 || need > 48 * 1024) {
+        if (npt == 0 || need > snn::SAMPLE_SMEM_DEFAULT) {
             const size_t smem = (size_t)s->c.Iw * 4 + (size_t)NI * 2 + 16;
             k_serve_chunk_wide<<<nl, SC_THREADS, smem, st>>>(s->c, s->d, sg.live, kk);
         } else {

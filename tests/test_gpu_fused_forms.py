@@ -179,3 +179,47 @@ def test_rec_gather_runs_of_one_step(B, NI, N, NO):
         fired += int(rh.sum())
     assert fired > 0
     net.close()
+
+
+FRESH = """
+import sys
+sys.path[:0] = [%r, %r]
+import numpy as np
+import test_gpu_parity as tp
+import test_gpu_serving as ts
+
+def workload(B, N, NI):
+    p, r, s, w = tp.synth.workload(B, N, NI)
+    return p, np.minimum(r * np.float32(4 * 784 / NI), np.float32(900)), s, w
+%s
+"""
+SERVE_ONE = """
+p, r, s, w = workload(3, 20, 6032)
+m = tp.snn()
+net = m.Network(p, w_init=w)
+srv = m.snn_serve_create(net.handle, 4, 1 << 30)
+ids = {m.snn_serve_submit(srv, r[q], int(s[q]), 30): q for q in range(3)}
+while m.snn_serve_status(srv)["active"] or m.snn_serve_status(srv)["queued"]:
+    m.snn_serve_step(srv, 11)
+m.snn_serve_wait(srv)
+for i, c in zip(*m.snn_serve_poll(srv, 20)):
+    assert np.array_equal(c, ts.alone_counts(p, w, 0, r[ids[int(i)]], int(s[ids.pop(int(i))]), 30))
+assert not ids
+"""
+
+
+@pytest.mark.parametrize("code", [
+    "for B in (104, 105, 107, 108): tp.parity_all_modes(*workload(B, 12, 2900), 4, modes=('graph',))",
+    "tp.parity_all_modes(*workload(1, 12, 3063), 4, learn=False, modes=('graph',))",
+    "for NI in (3997, 3998, 4007, 4008): tp.parity_all_modes(*workload(2, 20, NI), 6, learn=False, modes=('persistent',))",
+    SERVE_ONE,
+], ids=["column tiles", "column tiles, frozen", "sample per CTA", "serving"])
+def test_dynamic_shared_memory_near_the_default_limit(code):
+    """The default limit of 48 KB counts a kernel's static shared memory too. In a
+    fresh process each: a larger run of the same kernel raises the limit for good."""
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    q = subprocess.run([sys.executable, "-c", FRESH % (os.path.dirname(here), here, code)], capture_output=True, text=True)
+    assert q.returncode == 0, q.stderr[-2000:]
