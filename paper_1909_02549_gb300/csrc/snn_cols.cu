@@ -495,7 +495,12 @@ __global__ void __launch_bounds__(CT, CB) k_cols(const __grid_constant__ Consts 
 
 // Columns per block: eight (a 32-byte sector of each state row), unless four let
 // CB blocks share an SM's shared memory (their phases overlap: one streams state
-// while another updates) or give every SM two blocks; TC = 0: no tile fits.
+// while another updates) or give every SM two blocks and still fit one wave: a few
+// blocks left over take a second one (784->2000 at B = 16 and 128, us a step with
+// four columns, eight, and the separate kernels: 19.6, 13.4, 17.8 and 28.6, 19.5,
+// 33.7; frozen at B = 128: 11.6, 7.5, 11.7).  With the maximum, whose walk has more
+// registers and longer rows, two short waves stay faster above 512 samples (784->2200,
+// B = 1024: 210 and 275).  TC = 0: no tile fits.
 ColGeom col_geom(const Consts& c, int sms, size_t smem_optin) {
     ColGeom g{};
     g.Ip = (c.n_in + 7) & ~7;
@@ -516,7 +521,8 @@ ColGeom col_geom(const Consts& c, int sms, size_t smem_optin) {
         const size_t enc = up((size_t)ES * c.Iw * 4);
         if (t.smem < enc) t.smem = enc;
         if (t.smem + 1024 > smem_optin) continue;
-        if (g.TC == 0 || g.smem > share || g.ntile < 2 * sms) g = t;
+        const bool one_wave = t.ntile <= CB * sms || (c.learn && c.reduce == SNN_REDUCE_MAX && c.B > 512);
+        if (g.TC == 0 || g.smem > share || (g.ntile < 2 * sms && one_wave)) g = t;
         else break;
     }
     return g;

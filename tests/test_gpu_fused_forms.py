@@ -223,3 +223,13 @@ def test_dynamic_shared_memory_near_the_default_limit(code):
     here = os.path.dirname(os.path.abspath(__file__))
     q = subprocess.run([sys.executable, "-c", FRESH % (os.path.dirname(here), here, code)], capture_output=True, text=True)
     assert q.returncode == 0, q.stderr[-2000:]
+
+
+@pytest.mark.parametrize("B,NI,N,T,reduce", [
+    (3, 120, 1824, 12, "mean"),    # four columns a block: the widest layer whose blocks fit one wave
+    (3, 120, 1828, 12, "mean"),    # eight columns: four would need a second wave
+    (5, 120, 2031, 12, "sum"),     # the same with unaligned rows and a short last tile
+    (514, 100, 1900, 3, "max"),    # four again: the maximum above 512 samples
+])
+def test_column_tile_step_between_its_tiles(B, NI, N, T, reduce):
+    test_column_tile_step(B, NI, N, T, reduce)
