@@ -483,7 +483,9 @@ __global__ void __launch_bounds__(CT, CB) k_cols(const __grid_constant__ Consts 
                 if (nev + np[k] - (int)both[k] < B) D = fmaxf(D, 0.0f);   // idle samples add 0
             } else {
                 D = __fsub_rn(np[k] ? pt[k] : 0.0f, dep[k]);
-                if (RED == SNN_REDUCE_MEAN) D = batch_mean(c, D);
+                // 0 / B = 0 with its sign: no division for the columns without a trace
+                // (784->2440, B = 20: 22.8 -> 20.0 us a step; separate kernels 21.1)
+                if (RED == SNN_REDUCE_MEAN && D != 0.0f) D = batch_mean(c, D);
             }
             if (c.wmaster) master_add(wv[k], wl[k], D, c.w_min, c.w_max);
             else wv[k] = plain_add(wv[k], D, c.w_min, c.w_max);

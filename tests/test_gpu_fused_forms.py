@@ -233,3 +233,17 @@ def test_dynamic_shared_memory_near_the_default_limit(code):
 ])
 def test_column_tile_step_between_its_tiles(B, NI, N, T, reduce):
     test_column_tile_step(B, NI, N, T, reduce)
+
+
+def test_column_tile_step_mean_of_columns_without_a_trace():
+    """A batch that is no power of two, few columns firing: the mean of the other
+    columns' zero sums, and weights at both bounds, for both masters."""
+    import test_gpu_parity as tp
+    p, r, s, w = tp.synth.workload(7, 203, 120)
+    r = np.minimum(r * np.float32(20), np.float32(900))
+    w = np.where(np.arange(203) % 5 == 0, w, np.float32(0)).astype(np.float32)
+    w[:, 2::10] = 1.0
+    for wmaster in (0, 1):
+        p.update(wmaster=wmaster)
+        st, rec = tp.parity_all_modes(p, r, s, w, 60, modes=("graph", "step"))
+        assert rec.raster_e.sum() > 0 and (np.abs(st.w - w).max(0) == 0).any()
