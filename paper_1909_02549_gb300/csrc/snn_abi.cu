@@ -264,8 +264,8 @@ snn::Consts make_consts(const snn_net* n, int B, float dt, int learn, int reduce
 
 // One step of the per-step and graph forms: a launch over column tiles, or the
 // separate encode, neuron and update kernels where that does not apply (the
-// post-triggered rule, layers whose tile does not fit shared memory) and in
-// profiled runs, whose report counts them.
+// post-triggered rule, layers whose tile does not fit shared memory) or does not
+// pay (snn_cols.cu), and in profiled runs, whose report counts them.
 cudaError_t step_launches(const snn::Consts& c, const snn::Bufs& d, int t, int T, cudaStream_t s, snn::Prof* pp) {
     int used = 0;
     if (!pp) {

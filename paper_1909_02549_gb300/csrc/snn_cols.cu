@@ -530,6 +530,44 @@ ColGeom col_geom(const Consts& c, int sms, size_t smem_optin) {
     return g;
 }
 
+// Whether the column tiles are faster than the separate kernels.  A block runs all
+// samples of its columns, so few columns leave SMs idle when samples are many, and
+// it stages its weights before it starts, which few samples do not repay where the
+// blocks need several waves.  The separate update grows with n_in, B and the spikes,
+// so learning moves the line far out.  Us a step, graph runs of 40 steps, separate
+// kernels / this one (784 inputs: digits; 100: 120 Hz):
+//   frozen, aligned rows, 100 inputs: 50 columns at B = 128 and 1024: 7.0 / 5.4, 8.1 /
+//   27; 600 at 176 and 428 7.7 / 6.3, 8.5 / 11.2; 1800 at 64 and 128 7.4 / 6.7, 8.1 /
+//   8.5; 2440 at 512 19.7 / 17.3; 784 inputs: 50 at 256 and 1024 11 / 8.7, 16.8 / 25.7;
+//   600 at 428 and 2048 14.2 / 13.1, 44.8 / 51.2; 1600 at 1024 44.0 / 36.6; 32 inputs:
+//   1000 at B = 16, 64 and 428: 4.5 / 6.0, 4.8 / 4.2, 7.0 / 10.6;
+//   frozen, rows that are not 16-byte aligned, 784 inputs: 1023 at 100 and 128 10.4 /
+//   8.3, 10.6 / 13.5; 2999 at 48 and 100 10.2 / 9.6, 12.4 / 14.8;
+//   learning, several waves: 10000 columns at B = 33, 64 and 200: 784 inputs 47.8 /
+//   54.5, 57.7 / 47.2, 149.7 / 85; 100 inputs 19.0 / 28.9, 24.7 / 20.4, 57 / 43; 225
+//   inputs 15.5 / 28, 18.1 / 18.3, 39.0 / 39.4; unaligned, 784->6001 at 33, 64 and 128
+//   34.3 / 44.6, 42.8 / 44.9, 65.9 / 58; sum, 225->10000 at 33 and 64 13.9 / 15.7, 17.6 /
+//   16.7; max, 784->6400 at 40 64.6 / 54.2;
+//   learning, one wave: divided means of a few samples, 1023->2440 at B = 3 and 40 21.4 /
+//   24, 33.1 / 29.8; unaligned, 784->1537 at 33, 128 and 256 22.2 / 21, 31.2 / 35.6,
+//   52.5 / 49.2; 32 inputs, 1000 at B = 128 and 256 7.0 / 5.6, 7.7 / 9.6.
+bool pays(const Consts& c, const ColGeom& g, int sms) {
+    const bool aligned = (c.N & 3) == 0, waves = (c.N + 7) / 8 > CB * sms, few_inputs = c.n_in <= 96;
+    if (!c.learn) {
+        if (few_inputs) return false;
+        if (waves) return aligned && c.B >= 64;
+        if (g.TC == 8) return aligned ? c.N >= 16 * sms || c.n_in >= 512 || c.B <= 64 * c.Iw : c.B <= 48;
+        if (!aligned && c.N > 512) return c.B <= (c.N <= 8 * sms ? 100 : 64);
+        if (c.n_in >= 512 && c.N >= 1000) return true;
+        return c.B <= (c.N < 64 ? 80 + 12 * c.Iw : c.N <= 8 * sms ? 112 + 16 * c.Iw : 64 + 12 * c.Iw);
+    }
+    const bool divides = c.reduce == SNN_REDUCE_MEAN && !c.B_pow2;
+    if (few_inputs) return !waves && c.B <= (c.reduce == SNN_REDUCE_MAX ? 256 : 128) && (g.TC == 4 || !divides);
+    if (waves) return c.B >= (divides ? (c.n_in >= 512 ? 100 : 160) : aligned ? 40 : 128);
+    if (g.TC == 8) return !divides || c.n_in <= 128 || c.B > (aligned ? 12 : 31);
+    return aligned || c.N <= 8 * sms || c.n_in < 512 || c.B <= 48 || c.B >= 256;
+}
+
 }  // namespace
 
 cudaError_t launch_cols_step(const Consts& c, const Bufs& d, int t_local, int T, cudaStream_t s, int* used) {
@@ -541,11 +579,7 @@ cudaError_t launch_cols_step(const Consts& c, const Bufs& d, int t_local, int T,
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     ColGeom g = col_geom(c, sms, (size_t)optin);
-    // More tiles than one wave and few samples: a block then stages its weights
-    // for little work, and the separate kernels are faster (6400 columns at
-    // B = 1, 16 and 32: 20, 26 and 29 us a step against 22, 28 and 29;
-    // 1600 columns: 13, 18 and 19 against 9, 13 and 14).
-    if (g.TC == 0 || ((c.N + 7) / 8 > CB * sms && c.B <= 32)) return cudaSuccess;
+    if (g.TC == 0 || !pays(c, g, sms)) return cudaSuccess;
     const bool v4 = (c.N & 3) == 0;
     auto kern = c.reduce == SNN_REDUCE_SUM    ? (v4 ? k_cols<SNN_REDUCE_SUM, true> : k_cols<SNN_REDUCE_SUM, false>)
                 : c.reduce == SNN_REDUCE_MEAN ? (v4 ? k_cols<SNN_REDUCE_MEAN, true> : k_cols<SNN_REDUCE_MEAN, false>)

@@ -247,3 +247,47 @@ def test_column_tile_step_mean_of_columns_without_a_trace():
         p.update(wmaster=wmaster)
         st, rec = tp.parity_all_modes(p, r, s, w, 60, modes=("graph", "step"))
         assert rec.raster_e.sum() > 0 and (np.abs(st.w - w).max(0) == 0).any()
+
+
+@pytest.mark.parametrize("B,NI,N,T,reduce", [
+    (1, 97, 5, 40, "max"),         # the fewest inputs, fewer columns than a quad pair
+    (257, 100, 130, 12, "mean"),   # four columns a block, nine mask words, a last tile of two
+    (65, 120, 2504, 6, "max"),     # eight columns a block, three mask words
+    (130, 100, 3653, 4, "sum"),    # several waves, unaligned rows, a short last tile
+])
+def test_column_tile_step_from_97_inputs(B, NI, N, T, reduce):
+    test_column_tile_step(B, NI, N, T, reduce)
+
+
+@pytest.mark.parametrize("B,NI,N", [
+    (128, 100, 40), (129, 100, 40), (100, 100, 1001), (101, 100, 1001), (48, 97, 2441), (49, 97, 2441)])
+def test_frozen_steps_on_both_sides_of_the_tiles_line(B, NI, N):
+    import test_gpu_parity as tp
+    p, r, s, w = tp.synth.fig1_workload(B, N, n_in=NI)
+    st, rec = tp.parity_all_modes(p, r, s, w, 40, learn=False, modes=("graph", "step"))
+    assert rec.raster_e.sum() > 0
+
+
+@pytest.mark.parametrize("B,NI,N", [(4096, 100, 50), (2048, 225, 50)])
+def test_frozen_steps_of_many_samples_spread_over_the_gpu(B, NI, N):
+    """A few blocks that own the columns of all samples took four to eight times as
+    long as the separate kernels, which a profiled run launches."""
+    m = snn()
+    from paper_1909_02549_gb300 import synth
+    p, r, s, w = synth.fig1_workload(B, N, n_in=NI)
+    net = m.Network(p, w_init=w)
+    R, S = dev(r), dev(s)
+    best = {}
+    for profile in (False, True):
+        ms = []
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            e0.record()
+            net.run(R, S, 50, learn=False, mode="graph", profile=profile)
+            e1.record()
+            torch.cuda.synchronize()
+            ms.append(e0.elapsed_time(e1))
+        best[profile] = min(ms)
+    net.close()
+    assert best[False] < 1.5 * best[True], best
