@@ -49,11 +49,26 @@ __global__ void __launch_bounds__(1024, 1) k_infer(const __grid_constant__ Const
 cudaError_t launch_infer(const Consts& c, const Bufs& d, int T, cudaStream_t s, int* used) {
     *used = 0;
     const int npt = sample_npt(c.N);
-    // Above 4096 neurons a CTA's step takes as long as the column kernel's until
-    // the samples fill the SMs (6400 neurons, us a step, before and here: B = 1
-    // 6.6 and 6.7, B = 16 7.0 and 7.5, B = 152 11.0 and 7.4; FP8, whose decoding
-    // is repeated by every sample, B = 256 18.8 and 34).
-    if (npt == 8 && (c.B < 64 || c.wprec == SNN_W_FP8E4M3)) return cudaSuccess;
+    // Above 4096 neurons a CTA's step takes as long as the column kernel's of a whole
+    // batch until the samples fill the SMs, one each, and a second wave doubles its time:
+    // from 64 samples, and with a last wave at least five eighths full (784->6400, us a
+    // step there and here: B = 16, 64, 128, 160 and 256 7.0 / 7.5, 8.6 / 7.8, 11.2 / 8.0,
+    // 12.3 / 13.9, 15.3 / 14.7).  Not FP8, whose decoding is repeated by every sample
+    // (B = 256: 18.8 and 34).
+    // The weight rows come from L2 for each sample, so dense inputs favour the column
+    // kernel, more so the wider the layer.  The figures above and those in the header
+    // are at image rates (1 % of the inputs active); with an eighth active: 784->1000
+    // still faster at every B, 784->3000 B = 1 12.9 / 21.7, B = 64 31.4 / 22.3, 784->6400
+    // B = 64 and 128 27.8 / 40.9, 41.3 / 41.1.  The rates are on the device, so the rule
+    // does not look at them.
+    if (npt == 8) {
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        const bool short_wave = c.B > sms && 8 * ((c.B - 1) % sms + 1) < 5 * sms;
+        if (c.B < 64 || short_wave || c.wprec == SNN_W_FP8E4M3) return cudaSuccess;
+    }
     const size_t smem = sample_smem(c.n_in, c.Iw, true, c.rec_input != 0).bytes;
     if (c.learn || c.test_timeout || npt == 0 || c.n_in > 65535 || smem > 200 * 1024) return cudaSuccess;
     cudaError_t e;

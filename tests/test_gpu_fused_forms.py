@@ -291,3 +291,31 @@ def test_frozen_steps_of_many_samples_spread_over_the_gpu(B, NI, N):
         best[profile] = min(ms)
     net.close()
     assert best[False] < 1.5 * best[True], best
+
+
+@pytest.mark.parametrize("B,NI,N,wprec", [
+    (64, 60, 8192, 0), (64, 60, 8192, 1),      # the widest layer at eight neurons per thread
+    (65, 130, 5003, 0), (65, 130, 5003, 1),    # a ragged one
+    (70, 60, 4097, 2),                         # FP8: the column kernel
+    (153, 40, 4200, 0),                        # one sample past a wave: the column kernel
+    (247, 40, 4200, 1),                        # a second wave five eighths full
+])
+def test_learning_off_wide_layers(B, NI, N, wprec):
+    """Eight neurons per thread (64 samples and more) and its limits: a learning run, a
+    frozen run that continues it with traces to decay, and another learning one."""
+    import test_gpu_parity as tp
+    import oracle
+    import os
+    oracle.set_threads(os.cpu_count() or 1)
+    p, r, s, w = tp.synth.workload(B, N, NI)
+    r = np.minimum(r * np.float32(4 * 784 / NI), np.float32(900))
+    r2 = np.roll(r, 7, axis=1)
+    r2[0] = 0
+    net, st = None, None
+    for k, (rates, steps, learn, mode) in enumerate([(r, 3, True, "graph"), (r2, 25, False, "persistent"), (r, 2, True, "graph")]):
+        st, rec = tp.oracle_run(p, rates, s, w, steps, learn=learn, st=st, episodic=k == 0, wprec=wprec)
+        net, g = tp.gpu_run(p, rates, s, w, steps, learn=learn, mode=mode, net=net, continue_=k > 0, wprec=wprec)
+        tp.assert_parity(g, st, rec)
+        assert k != 1 or rec.raster_e.sum() > 0
+    net.close()
+    oracle.set_threads(1)
