@@ -452,9 +452,17 @@ cudaError_t launch_small(const Consts& c, const Bufs& d, int T, cudaStream_t s, 
     // steps, 512 and 8 629, 256 and 4 709; 784->400, B = 16: 1024 threads 1441,
     // 512 1915).  Above ITEMS items a CTA the column kernel is faster (us a step
     // there and here, 1000 columns of 100 inputs at B = 4 and 8: 9.9 and 10.8,
-    // 6.7 and 11.7; 784->400 at B = 16: 8.6 and 5.3).
+    // 6.7 and 11.7; 784->400 at B = 16: 8.6 and 5.3).  Without lateral inhibition the
+    // columns fire in bursts, and each that fired costs a warp a pass over its rows, with
+    // a division each where the mean takes one: fewer items (100 inputs of 120 Hz: 100->
+    // 224, B = 32 9.2 and 10.5, 100->6400, B = 1 9.6 and 12.2, 100->280, B = 24 10.3 and
+    // 12.8, 100->144, B = 24 10.3 and 10.8; but 100->100, B = 32 9.1 and 8.8, 100->4000, B
+    // = 1 9.3 and 7.8, 100->100, B = 17 10.2 and 9.0).  With inhibition, dense inputs cost
+    // the rows' passes too: 784->448, B = 16 at 1 and 6 % active 9.3 and 6.4, 15.8 and 19.8.
     constexpr size_t SMEM = 224 * 1024;
-    constexpr int ITEMS = 448;
+    const bool inhibition = c.w_ei != 0.0f && c.w_ie != 0.0f;
+    const bool divides = c.reduce == SNN_REDUCE_MEAN && !c.B_pow2;
+    const int ITEMS = inhibition ? 448 : divides && c.B > 16 ? 168 : 288;
     const bool few = c.B <= 4;
     using Kern = void (*)(Consts, Bufs, SmallGeom, int);
     static const Kern kerns[3][2] = {{k_small<1024, 1, false>, k_small<1024, 1, true>},

@@ -319,3 +319,16 @@ def test_learning_off_wide_layers(B, NI, N, wprec):
         assert k != 1 or rec.raster_e.sum() > 0
     net.close()
     oracle.set_threads(1)
+
+
+@pytest.mark.parametrize("B,NI,N,reduce", [
+    (32, 100, 144, "mean"), (32, 100, 145, "mean"),    # 288 items a CTA, and more: the column kernel
+    (24, 60, 112, "mean"), (24, 60, 113, "mean"),      # divided means: 168
+    (14, 40, 256, "max"), (1, 40, 4608, "sum"), (1, 40, 4609, "sum"),
+])
+def test_small_batch_without_inhibition(B, NI, N, reduce):
+    import test_gpu_parity as tp
+    p, r, s, w = tp.synth.fig1_workload(B, N, n_in=NI)
+    r = r * np.float32(100 / NI)
+    st, rec = tp.parity_all_modes(p, r, s, w, 60, reduce=reduce, modes=("persistent",))
+    assert rec.raster_e.sum() > 0 and np.abs(st.w - w).max() > 0
