@@ -31,12 +31,16 @@
 // separate neuron passes', the quiet-column pass's, the encode's or the first STDP
 // pass's around its calls: the step's code does not fit the instruction cache (92 % of
 // its requests hit at 784->6400, 74 % at 784->100 with the post-triggered rule), and
-// unrolled it was half as large again.  The step's start is unrolled in the narrow
-// instantiation only.  Per step, all unrolled / so: 784->6400, B = 256 30.5 / 29.7 us;
-// 784->400, B = 1024 33.1 / 32.8; 784->100, B = 64, rule, max 13.3 / 11.7; 225->290, B =
-// 644 17.8 / 17.4; 1023->426, B = 608 35.5 / 35.7; 784->321, B = 115, FP8, max 14.4 /
-// 14.2; 100->1000, B = 1024 59.8 / 60.0; 100->10000, B = 256 64.8 / 64.9.  (All rolled:
-// 29.6, 32.7, 11.8, 18.2, 35.9, 14.5, 60.8, 65.7.)
+// unrolled it was half as large again.  The step's start, and the neuron phase's loop
+// over the rows past the staged pairs, are unrolled in the narrow instantiation only.
+// Us a step, all unrolled / so (digits, pair rule, mean unless said; runs of 100 steps,
+// of 250 at 784->400 and with the rule): 784->6400, B = 256 33.5 / 32.8; 784->400, B =
+// 1024 31.6 / 31.2; 784->100, B = 64, rule, max 13.3 / 11.7; 225->290, B = 644 17.9 /
+// 17.5; 1023->426, B = 608 37.0 / 36.6; 1023->150, B = 1024 36.5 / 36.1 (with those rows
+// rolled 37.0); 784->321, B = 115, FP8, max 16.1 / 15.9; 100->300, B = 300 and 600 13.6 /
+// 13.5, 14.8 / 15.1, which no variant of these loops changes.  1000 steps of 100 inputs
+// at 120 Hz: 1000 columns, B = 1024 73.6 / 73.2; 10000, B = 16 17.6 / 17.2; 250 steps,
+// 10000, B = 256 70.0 / 70.0.
 #include <cfloat>
 #include <mutex>
 
@@ -1120,6 +1124,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t ta, const uint32_t (&r)[16]) 
 // order, as the per-step kernels.  Inlined: a call would have to save the
 // kernel's live values around it, through L1 that the shared memory leaves
 // small.
+template <bool NARROW>
 __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, const float* Ws, float* Es,
                                           const float* wsc, int ncmax, const uint32_t* actN,
                                           const uint16_t* actS, int caps, uint32_t* Qm, uint32_t* Sm,
@@ -1154,7 +1159,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
                         I2 = __fadd_rn(__fadd_rn(I2, w.z), v.z);
                         I3 = __fadd_rn(__fadd_rn(I3, w.w), v.w);
                     }
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
                     for (; a < na; ++a) {
                         const int r = a < ns ? (int)al[a] : (int)__ldcg(&ag[a]);
                         const float4 w = *(const float4*)(wc + r * nst);
@@ -1174,7 +1179,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
                         I2 = __fadd_rn(__fadd_rn(I2, w_read_bf16(w.z)), w_read_bf16(v.z));
                         I3 = __fadd_rn(__fadd_rn(I3, w_read_bf16(w.w)), w_read_bf16(v.w));
                     }
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
                     for (; a < na; ++a) {
                         const int r = a < ns ? (int)al[a] : (int)__ldcg(&ag[a]);
                         const float4 w = *(const float4*)(wc + r * nst);
@@ -1198,7 +1203,7 @@ __device__ __forceinline__ void neuron_phase(const Consts& c, const Bufs& d, con
                         I2 = __fadd_rn(__fadd_rn(I2, w_read_e4m3(w.z, v2)), w_read_e4m3(u.z, v2));
                         I3 = __fadd_rn(__fadd_rn(I3, w_read_e4m3(w.w, v3)), w_read_e4m3(u.w, v3));
                     }
-#pragma unroll 1
+#pragma unroll(NARROW ? 4 : 1)
                     for (; a < na; ++a) {
                         const int r = a < ns ? (int)al[a] : (int)__ldcg(&ag[a]);
                         const float4 w = *(const float4*)(wc + r * nst);
@@ -1611,7 +1616,7 @@ k_persistent(const __grid_constant__ Consts c, const __grid_constant__ Bufs d, c
         __syncthreads();
 
         if (FUSED) {
-            neuron_phase(c, d, Ws, Es, wsc, L.ncmax, actN, actS, caps, Qm, Sm, cntS, thj, tq, tstate, nc, nst,
+            neuron_phase<NARROW>(c, d, Ws, Es, wsc, L.ncmax, actN, actS, caps, Qm, Sm, cntS, thj, tq, tstate, nc, nst,
                          j0, cur, t, p3);
         } else {
             if (NARROW) synaptic_currents_narrow(c, d, Ws, Es, wsc, L.ncmax, actN, actS, caps, nc, nst, cur);

@@ -332,3 +332,15 @@ def test_small_batch_without_inhibition(B, NI, N, reduce):
     r = r * np.float32(100 / NI)
     st, rec = tp.parity_all_modes(p, r, s, w, 60, reduce=reduce, modes=("persistent",))
     assert rec.raster_e.sum() > 0 and np.abs(st.w - w).max() > 0
+
+
+@pytest.mark.parametrize("wprec", [0, 1, 2])
+def test_narrow_column_kernel_rows_past_the_staged_ones(wprec):
+    """One column a CTA, samples with hundreds of active inputs (odd and even counts):
+    most of a sample's rows come from the list's part that is not staged."""
+    import test_gpu_parity as tp
+    B, NI, N = 600, 1023, 130
+    p, r, s, w = tp.synth.workload(B, N, NI)
+    r = np.minimum(r * np.float32(12), np.float32(900))
+    st, rec = tp.parity_all_modes(p, r, s, w, 6, reduce="sum", modes=("persistent",), wprec=wprec)
+    assert rec.raster_e.sum() > 0 and (r > 0).sum(1).max() > 300
