@@ -1528,6 +1528,13 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
     geom.nd = sample_tiles * geom.ntn_drive;
     const int last = geom.nd % pairs;      // drive tiles of the round that is not full
     geom.parts = 4 * last + ro_items <= pairs ? 4 : 2 * last + ro_items <= pairs ? 2 : 1;
+    // half as many where 32 items and more would read the few rows of a small S: all of
+    // them ask for the same lines at the same time (us a step, 60 steps, in the finer
+    // parts / so: 64->4096 at B = 1, 8 and 15 37.2 / 30.1, 35.1 / 26.5, 37.8 / 31.7,
+    // 1024->4096 at B = 1 and 12 46.7 / 38.0, 40.9 / 32.1, 64->8192 at B = 4 70.5 / 62.2;
+    // from 128 KB on the finer ones: 1024->4096, B = 15 22.7 / 25.7; with 16 items too:
+    // 64->1000, B = 1 13.5 / 15.0)
+    if (geom.parts * last >= 32 && (size_t)B * r->K * 2 < 128 * 1024) geom.parts = std::max(1, geom.parts / 2);
     geom.nfull = geom.nd - last;
     geom.nitems = geom.nfull + geom.parts * last + ro_items;
     const unsigned dgrid = 2u * (unsigned)std::min(geom.nitems, pairs);   // a pair of CTAs per item

@@ -344,3 +344,10 @@ def test_narrow_column_kernel_rows_past_the_staged_ones(wprec):
     r = np.minimum(r * np.float32(12), np.float32(900))
     st, rec = tp.parity_all_modes(p, r, s, w, 6, reduce="sum", modes=("persistent",), wprec=wprec)
     assert rec.raster_e.sum() > 0 and (r > 0).sum(1).max() > 300
+
+
+@pytest.mark.parametrize("B,NI,N", [(1, 64, 2048), (2, 33, 4000), (9, 30, 7700)])
+def test_rec_tensor_form_of_a_few_samples_in_coarser_parts(B, NI, N):
+    """Wide layers whose operand is small: halves instead of quarters, whole tiles
+    instead of halves."""
+    test_rec_tensor_form_cut_tiles(B, NI, N, 10)
