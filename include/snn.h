@@ -500,10 +500,11 @@ enum {
     SNN_REC_KERNEL_ENCODE = 0,   /* Poisson input spikes */
     SNN_REC_KERNEL_DRIVE = 1,    /* drive and neuron update (gather or tensor form) */
     SNN_REC_KERNEL_READOUT = 2,  /* summed readout */
-    SNN_REC_KERNEL_COUNT = 3
+    SNN_REC_KERNEL_COUNTS = 3,   /* tensor form: spike counts, every 31 steps */
+    SNN_REC_KERNEL_COUNT = 4
 };
 /* Device time of the last run made with SNN_PROFILE (every step's launches
- * bracketed by CUDA events: up to 6*T events, created once and kept by the
+ * bracketed by CUDA events: up to 8*T events, created once and kept by the
  * network), per kernel class: ms[k] summed milliseconds,
  * launches[k] launches, k < count <= SNN_REC_KERNEL_COUNT.  Synchronises.
  * Errors: SNN_ERR_ARG, SNN_ERR_STATE (last run not profiled), SNN_ERR_CUDA. */

@@ -1562,7 +1562,9 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
         mark(SNN_REC_KERNEL_DRIVE, false);
         if (dense && (!d.hist || geom.slot == HIST - 1 || t == T - 1)) {
             const size_t warps = (size_t)((B + 31) / 32) * c.Nw;
+            mark(SNN_REC_KERNEL_COUNTS, true);
             k_rec_fold<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(c, d, t, geom.slot + 1);
+            mark(SNN_REC_KERNEL_COUNTS, false);
         }
         // the tensor form's product adds each step's readout one step later;
         // the run's last step is read out here

@@ -96,7 +96,7 @@ class snn_rec_spec(C.Structure):
 SNN_REC_GATHER = 1 << 8      # exact gather form of the drive
 SNN_REC_TENSOR = 1 << 9      # dense tensor-core form
 REC_FORMS = {"auto": 0, "gather": SNN_REC_GATHER, "tensor": SNN_REC_TENSOR}
-REC_KERNELS = ("encode", "drive", "readout")
+REC_KERNELS = ("encode", "drive", "readout", "counts")
 REC_FIELDS = {"v": SNN_REC_V, "i_syn": SNN_REC_I_SYN, "spikes": SNN_REC_SPIKES,
               "counts": SNN_REC_COUNTS, "v_out": SNN_REC_V_OUT, "raster": SNN_REC_RASTER,
               "raster_input": SNN_REC_RASTER_INPUT, "step": SNN_REC_STEP}

@@ -351,3 +351,15 @@ def test_rec_tensor_form_of_a_few_samples_in_coarser_parts(B, NI, N):
     """Wide layers whose operand is small: halves instead of quarters, whole tiles
     instead of halves."""
     test_rec_tensor_form_cut_tiles(B, NI, N, 10)
+
+
+@pytest.mark.parametrize("T,folds", [(1, 1), (31, 1), (32, 2), (62, 2), (63, 3)])
+def test_rec_profile_brackets_the_spike_counts(T, folds):
+    p, r, s, wf, wr, wo = dyadic_workload(4, 64, 96, 10, seed=23)
+    net = snn().RecNetwork(p, wf, wr, wo)
+    for form, n in (("tensor", folds), ("gather", 0)):
+        net.run(dev(r), dev(s), T, form=form, profile=True)
+        prof = net.profile()
+        assert prof["counts"][1] == n and (prof["counts"][0] > 0) == (n > 0), prof
+        assert prof["drive"][1] == T
+    net.close()
