@@ -363,3 +363,27 @@ def test_rec_profile_brackets_the_spike_counts(T, folds):
         assert prof["counts"][1] == n and (prof["counts"][0] > 0) == (n > 0), prof
         assert prof["drive"][1] == T
     net.close()
+
+
+@pytest.mark.parametrize("N,wprec", [(1000, 0), (1000, 2), (3000, 0), (3000, 1), (5000, 0), (8200, 0), (8200, 1)])
+def test_serving_wider_layers(N, wprec):
+    """Two, four and eight neurons per thread, and the kernel of the layers too wide
+    for registers: requests of several calls with retirements inside them."""
+    import test_gpu_serving as ts
+    from paper_1909_02549_gb300 import synth
+    m, NI, nreq = snn(), 100, 7
+    p, r, s, w = synth.workload(nreq, N, NI)
+    r = np.minimum(r * np.float32(30), np.float32(900))
+    net = m.Network(p, w_init=w, wprec=wprec)
+    srv = m.snn_serve_create(net.handle, 3, 1 << 30)
+    ids = {m.snn_serve_submit(srv, r[q], int(s[q]), 21 + 5 * q): q for q in range(nreq)}
+    while m.snn_serve_status(srv)["active"] or m.snn_serve_status(srv)["queued"]:
+        m.snn_serve_step(srv, 8)
+    m.snn_serve_wait(srv)
+    done, counts = m.snn_serve_poll(srv, N, max_n=nreq)
+    m.snn_serve_destroy(srv)
+    assert sorted(int(i) for i in done) == sorted(ids) and counts.sum() > 0
+    for i, c in zip(done, counts):
+        q = ids[int(i)]
+        assert np.array_equal(c, ts.alone_counts(p, w, wprec, r[q], int(s[q]), 21 + 5 * q)), q
+    net.close()
