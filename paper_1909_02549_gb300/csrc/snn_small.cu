@@ -508,7 +508,12 @@ cudaError_t launch_small(const Consts& c, const Bufs& d, int T, cudaStream_t s, 
         g = t;
         if (t.ncc <= 32) break;
     }
-    if (g.CS == 0) return cudaSuccess;
+    // A run's start costs more here (a few CTAs load the weights and list the live inputs,
+    // a word after the other), which some steps repay: us a run, there and here, at T = 1,
+    // 3 and 10: 784->100, B = 1 37 / 43, 51 / 46, 104 / 57; 784->1000, B = 1 43 / 71, 61 /
+    // 75, 134 / 91; 784->400, B = 16 40 / 53, 56 / 62, 117 / 102; 3000->50, B = 4 45 / 92,
+    // 76 / 118, 181 / 183; 100->4000, B = 1 38 / 52, 54 / 62, 112 / 100.
+    if (g.CS == 0 || T < 4 + (c.Iw + g.ncc) / 16) return cudaSuccess;
     cfg.blockDim = dim3(few ? 512 : 1024);                 // half of them neuron threads
     cfg.gridDim = dim3(g.CS);
     at[0].val.clusterDim.x = g.CS;

@@ -387,3 +387,19 @@ def test_serving_wider_layers(N, wprec):
         q = ids[int(i)]
         assert np.array_equal(c, ts.alone_counts(p, w, wprec, r[q], int(s[q]), 21 + 5 * q)), q
     net.close()
+
+
+@pytest.mark.parametrize("B,NI,N", [(1, 120, 60), (5, 784, 300)])
+def test_small_batch_runs_of_a_few_steps(B, NI, N):
+    """Continuing runs of one to nine steps, the column kernel's and the cluster's."""
+    import test_gpu_parity as tp
+    p, r, s, w = tp.synth.workload(B, N, NI)
+    r = np.minimum(r * np.float32(4 * 784 / NI), np.float32(900))
+    net, st, fired = None, None, 0
+    for k, T in enumerate((1, 2, 3, 4, 5, 6, 7, 8, 9, 30, 1)):
+        st, rec = tp.oracle_run(p, r, s, w, T, st=st, episodic=k == 0)
+        net, g = tp.gpu_run(p, r, s, w, T, mode="persistent", net=net, continue_=k > 0)
+        tp.assert_parity(g, st, rec)
+        fired += int(rec.raster_e.sum())
+    assert fired > 0
+    net.close()
