@@ -550,8 +550,11 @@ ColGeom col_geom(const Consts& c, int sms, size_t smem_optin) {
 //   16.7; max, 784->6400 at 40 64.6 / 54.2;
 //   learning, one wave: divided means of a few samples, 1023->2440 at B = 3 and 40 21.4 /
 //   24, 33.1 / 29.8; unaligned, 784->1537 at 33, 128 and 256 22.2 / 21, 31.2 / 35.6,
-//   52.5 / 49.2; 32 inputs, 1000 at B = 128 and 256 7.0 / 5.6, 7.7 / 9.6.
-bool pays(const Consts& c, const ColGeom& g, int sms) {
+//   52.5 / 49.2; 32 inputs, 1000 at B = 128 and 256 7.0 / 5.6, 7.7 / 9.6;
+//   runs of one step, which launch the drawing blocks on their own: 784->6400, B = 64 40.5
+//   / 44.6 learning, 35.8 / 38.1 frozen; B = 256 0.78 and 0.85 of the separate kernels'.
+bool pays(const Consts& c, const ColGeom& g, int sms, int T) {
+    if (T == 1 && c.N > 1024 && c.B < 128) return false;
     const bool aligned = (c.N & 3) == 0, waves = (c.N + 7) / 8 > CB * sms, few_inputs = c.n_in <= 96;
     if (!c.learn) {
         if (few_inputs) return false;
@@ -579,7 +582,7 @@ cudaError_t launch_cols_step(const Consts& c, const Bufs& d, int t_local, int T,
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     ColGeom g = col_geom(c, sms, (size_t)optin);
-    if (g.TC == 0 || !pays(c, g, sms)) return cudaSuccess;
+    if (g.TC == 0 || !pays(c, g, sms, T)) return cudaSuccess;
     const bool v4 = (c.N & 3) == 0;
     auto kern = c.reduce == SNN_REDUCE_SUM    ? (v4 ? k_cols<SNN_REDUCE_SUM, true> : k_cols<SNN_REDUCE_SUM, false>)
                 : c.reduce == SNN_REDUCE_MEAN ? (v4 ? k_cols<SNN_REDUCE_MEAN, true> : k_cols<SNN_REDUCE_MEAN, false>)

@@ -403,3 +403,16 @@ def test_small_batch_runs_of_a_few_steps(B, NI, N):
         fired += int(rec.raster_e.sum())
     assert fired > 0
     net.close()
+
+
+@pytest.mark.parametrize("B,NI,N", [(64, 100, 1028), (128, 100, 1028)])
+def test_column_tile_step_runs_of_one_step(B, NI, N):
+    import test_gpu_parity as tp
+    p, r, s, w = tp.synth.fig1_workload(B, N, n_in=NI)
+    net, st = None, None
+    for k, T in enumerate((40, 1, 1, 2, 1)):
+        st, rec = tp.oracle_run(p, r, s, w, T, st=st, episodic=k == 0)
+        net, g = tp.gpu_run(p, r, s, w, T, mode=("graph", "step")[k & 1], net=net, continue_=k > 0)
+        tp.assert_parity(g, st, rec)
+        assert k > 0 or rec.raster_e.sum() > 0
+    net.close()
