@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(32 * (GNW_MAX + GE), 1) k_rec_gather(RecConsts
 // kernels then run).  Clusters as wide as the SMs allow while a CTA keeps at
 // least 256 neurons: a wider cluster shares the row loads among more SMs but
 // not their latency.  Then the narrowest vector that GNW_MAX warps cover.
-GatherPlan gather_plan(const RecConsts& c, int sms) {
+GatherPlan gather_plan(const RecConsts& c, int sms, int T) {
     GatherPlan g{};
     if ((long long)c.n_in + c.N > 65535) return g;         // 16-bit row indices (the zero row's included)
     int cs = 1;
@@ -584,9 +584,11 @@ GatherPlan gather_plan(const RecConsts& c, int sms) {
     g.o_thr = up(g.o_lst + (size_t)(c.n_in + c.N + 40) * 2);
     g.smem = g.o_thr + (size_t)c.n_in * 4;
     if (g.smem > 224 * 1024) return g;
-    // the cluster barrier's acquire drops L1, so W_out is kept in shared memory where it fits
+    // the cluster barrier's acquire drops L1, so W_out is kept in shared memory where it fits;
+    // one step reads few of its rows (1024->4096, B = 16: 82.6 us with all of it copied, 56
+    // without, 69 in the per-step kernels)
     const size_t wo = up((size_t)(c.N + 1) * c.n_out * 2);
-    if (up(g.smem) + wo <= 224 * 1024) {
+    if (T > 1 && up(g.smem) + wo <= 224 * 1024) {
         g.o_wo = up(g.smem);
         g.smem = g.o_wo + wo;
     }
@@ -1543,7 +1545,7 @@ snn_status snn_rec_run(snn_rec* r, const float* rates, const uint64_t* seeds, in
     const bool fuse_enc = dense && !c.rec_input;
     // the gather form: all steps in one launch where its limits hold (a profiled
     // run keeps the per-step launches that its report counts)
-    const GatherPlan plan = dense || profile || T == 0 ? GatherPlan{} : gather_plan(c, r->num_sms);
+    const GatherPlan plan = dense || profile || T == 0 ? GatherPlan{} : gather_plan(c, r->num_sms, T);
     if (plan.CS) REC_TRY(r, launch_gather(c, d, plan, T, r->dev_err, st));
     for (int t = 0; t < (plan.CS ? 0 : T); ++t) {
         if (!fuse_enc || t == 0) {
