@@ -330,7 +330,14 @@ def sweep_point(snn, torch, flush, B, N, T, mode, reduce, learn, reps=3, warm=2,
             "weights": ("fp32", "bf16", "fp8")[wprec], "tuned_choice": chosen, "form_taken": taken,
             "ms_per_presentation": ms, "sample_timesteps_per_s": B * T / (ms * 1e-3),
             "roofline_frac": per * B * T / (ms * 1e-3) / peaks()["hbm_gbs"] / 1e9,
-            "kernel_ms": prof}
+            "kernel_ms": prof,
+            **({"kernel_ms_note": SEPARATE_KERNELS} if taken in (snn.SNN_MODE_STEP, snn.SNN_MODE_GRAPH) else {})}
+
+
+# A profiled run of the step and graph forms reports these; an unprofiled one takes the
+# column-tile kernel where that is faster, in less time than they add up to.
+SEPARATE_KERNELS = ("of the separate encode, neuron and update kernels, which a profiled step or graph "
+                    "run launches; the timed runs take the column-tile kernel where it is faster")
 
 
 def sweep_leg(a):
@@ -652,6 +659,14 @@ def recorded_profile(a, dom):
     return profile_record(PERSISTENT_PROFILE, KERNEL_SOURCES)
 
 
+def kernel_name(dom, B, learn):
+    """The kernel of a profile's class; the persistent form's launch is another kernel
+    for frozen runs and may be one for small batches."""
+    if dom != "persistent" or (learn and B > 32):
+        return "k_" + dom
+    return "k_small or k_persistent" if learn else "k_infer or k_persistent"
+
+
 def profile_roofline(a, net, snn, flush, run, restore, B, N, T, learn):
     """Dominant kernel's achieved algorithmic bandwidth from an event-bracketed pass."""
     try:
@@ -694,7 +709,8 @@ def profile_roofline(a, net, snn, flush, run, restore, B, N, T, learn):
                        "note": "the DRAM traffic is a small fraction of the algorithmic bytes "
                                "(the state stays on chip); issue slots and latency bound the "
                                "kernel", "source": rec_source}
-        return {"bound": "hbm", "kernel": "k_" + dom, "achieved": achieved, "peak": pk["hbm_gbs"],
+        separate = {"kernel_note": SEPARATE_KERNELS} if dom in ("encode", "neuron", "stdp") and not a.mode.startswith("tensor") else {}
+        return {"bound": "hbm", "kernel": kernel_name(dom, B, learn), "achieved": achieved, "peak": pk["hbm_gbs"],
                 "unit": "GB/s", "frac": achieved / pk["hbm_gbs"], "traffic": traffic,
                 "traffic_source": rec_source, "limiter": limiter,
                 "peak_source": pk["source"] + " hbm_gbs (burst copy), of measured",
@@ -704,7 +720,7 @@ def profile_roofline(a, net, snn, flush, run, restore, B, N, T, learn):
                 "avg_launch_us": avg_s * 1e6,
                 "share_of_device_time": dom_ms / prof_total if prof_total else None,
                 "kernel_ms_per_run": {k: v[0] / n_prof for k, v in agg.items() if v[1]},
-                "launches_per_run": {k: v[1] // n_prof for k, v in agg.items() if v[1]}}
+                "launches_per_run": {k: v[1] // n_prof for k, v in agg.items() if v[1]}, **separate}
     except Exception as e:                       # report, never hide the headline number
         return {"bound": "hbm", "achieved": None, "peak": None, "unit": "GB/s", "frac": None,
                 "traffic": None, "error": str(e)[:300]}
@@ -1016,6 +1032,12 @@ def rec_bytes_per_launch(p, B):
             + 2.0 * B * K + 2.0 * N * K + 2.0 * n_out * N + 8.0 * B * n_out)
 
 
+def rec_drive_bytes_per_launch(p, B):
+    """The drive kernel's share of ``rec_bytes_per_launch``: the spike counts' 8 bytes a
+    neuron and sample are moved by the counts' own kernel, once in 31 steps."""
+    return rec_bytes_per_launch(p, B) - 8.0 * B * p["n_hid"]
+
+
 def rec_leg(a):
     """The recurrent inference network at its full size: B = 4096 samples,
     T = 500 steps of 1 ms, bfloat16 weights.  Both forms of the drive: the
@@ -1068,7 +1090,7 @@ def rec_leg(a):
     # neuron) over all n_in + n_hid inputs, and the readout over the hidden ones
     # (zeros of W_rec and of the spike operand included)
     flop_launch = 2.0 * B * p["n_hid"] * K + 2.0 * B * p["n_out"] * p["n_hid"]
-    bytes_launch = rec_bytes_per_launch(p, B)
+    bytes_launch = rec_drive_bytes_per_launch(p, B)
     drive_ms, drive_n = prof["drive"]
     drive_s = drive_ms * 1e-3 / drive_n
     drive_gbs = bytes_launch / drive_s / 1e9
@@ -1088,7 +1110,7 @@ def rec_leg(a):
                          "achieved": drive_gbs, "peak": pk["hbm_gbs"], "unit": "GB/s",
                          "frac": drive_gbs / pk["hbm_gbs"],
                          "traffic": traffic, "traffic_source": traffic_src,
-                         "note": "%.1f MB per launch (state, operands, thresholds, S and W once) / "
+                         "note": "%.1f MB per launch (voltages and currents, operands, thresholds, S and W once) / "
                                  "%.1f us (CUDA events around each of the %d launches of a "
                                  "profiled presentation); peak: measured copy bandwidth"
                                  % (bytes_launch / 1e6, 1e6 * drive_s, drive_n),

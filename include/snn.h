@@ -85,7 +85,13 @@ typedef enum { SNN_W_FP32 = 0, SNN_W_BF16 = 1, SNN_W_FP8E4M3 = 2 } snn_wprec;
                                          copies them on the stream (pinned memory makes
                                          the copy asynchronous) */
 #define SNN_PROFILE         (1u << 4) /* bracket every kernel launch of the run with CUDA
-                                         events; read the times with snn_profile */
+                                         events; read the times with snn_profile.  Step and
+                                         graph runs then launch the separate encode, neuron
+                                         and update kernels, and the recurrent gather its
+                                         kernels of one step, so that the report has their
+                                         parts: same results, but other kernels, and more
+                                         time, than the run without this flag where that
+                                         fuses a step or a run into one launch */
 #define SNN_TEST_BARRIER_TIMEOUT (1u << 5) /* test only: the persistent kernel's first grid
                                          barrier waits for an arrival that never comes, so
                                          its bounded wait (a few ms here) runs out and the run
@@ -93,10 +99,16 @@ typedef enum { SNN_W_FP32 = 0, SNN_W_BF16 = 1, SNN_W_FP8E4M3 = 2 } snn_wprec;
 #define SNN_TENSOR_GATHER   (1u << 6) /* with SNN_MODE_TENSOR: sum the synaptic current over
                                          the active inputs in ascending order (exact) instead
                                          of the tensor-core product; the update stays a product */
-#define SNN_MODE_STEP       (0u << 8) /* one kernel launch per phase per time step */
+#define SNN_MODE_STEP       (0u << 8) /* kernel launches per time step: one over column
+                                         tiles where that is faster (pair rule), else one
+                                         per phase */
 #define SNN_MODE_GRAPH      (1u << 8) /* the T-step launch sequence captured once as a
                                          CUDA graph and replayed */
-#define SNN_MODE_PERSISTENT (2u << 8) /* one persistent cooperative kernel for all T steps */
+#define SNN_MODE_PERSISTENT (2u << 8) /* one launch for all T steps: a cooperative kernel in
+                                         which a CTA owns weight columns; a CTA per sample
+                                         with learning off; one thread-block cluster for a
+                                         few samples learning.  Takes what the cooperative
+                                         kernel's shared memory takes */
 #define SNN_MODE_AUTO       (3u << 8) /* library picks the mode (see snn_tune) */
 #define SNN_MODE_TENSOR     (4u << 8) /* per-step launches, captured as a CUDA graph, in which
                                          the synaptic current (Sec. "Implementation": the
@@ -273,7 +285,9 @@ SNN_API snn_status snn_write_weights(snn_net* net, const float* src, size_t byte
  * one stream).  Not thread-safe per server. */
 typedef struct snn_server snn_server;
 
-/* Device bytes of one slot's state (what admission counts against the cap). */
+/* Bytes of one slot (what admission counts against the cap): its state on the
+ * device, and two result rows and its share of three calls' lists and rates in
+ * pinned host memory that the kernels read and write. */
 SNN_API size_t snn_serve_slot_bytes(const snn_net* net);
 
 /* Create a server for net.  Errors: SNN_ERR_ARG, SNN_ERR_CAPACITY (the cap
@@ -290,14 +304,14 @@ SNN_API snn_status snn_serve_submit(snn_server* server, const float* rates_hz, u
 /* Admit queued requests into free slots, enqueue up to k steps of every
  * active slot on cuda_stream (fewer if all active presentations end sooner;
  * *steps_run, if not NULL, receives the number), and retire the slots whose
- * presentation ends within them; their spike counts are copied to the host
- * behind the steps.  Returns once the work is enqueued; it waits only when the
- * call three calls back has not yet finished on the device (its host staging
- * is reused), which bounds how far the host runs ahead.  Errors: SNN_ERR_ARG,
- * SNN_ERR_CUDA. */
+ * presentation ends within them; the kernel writes their spike counts to pinned
+ * host rows with its last steps.  Returns once the work is enqueued; it waits only
+ * when the call three calls back has not yet finished on the device (its pinned
+ * lists are reused), which bounds how far the host runs ahead, or when every result
+ * row is in use.  Errors: SNN_ERR_ARG, SNN_ERR_CUDA. */
 SNN_API snn_status snn_serve_step(snn_server* server, int k, void* cuda_stream, int* steps_run);
 
-/* Drain up to max finished requests whose counts have reached the host: ids
+/* Drain up to max finished requests whose call has ended on the device: ids
  * [max], excitatory spike counts [max][n_exc] (host); *n_out receives how
  * many were written.  Does not wait. */
 SNN_API snn_status snn_serve_poll(snn_server* server, uint64_t* ids, uint32_t* counts, int max,
@@ -308,7 +322,7 @@ SNN_API snn_status snn_serve_poll(snn_server* server, uint64_t* ids, uint32_t* c
 SNN_API snn_status snn_serve_wait(snn_server* server);
 
 /* Slots, active slots, queued requests, and retired-but-unpolled requests
- * (including those whose counts are still being copied); any may be NULL. */
+ * (including those whose call is still running); any may be NULL. */
 SNN_API snn_status snn_serve_status(const snn_server* server, int* slots, int* active,
                                     int* queued, int* done);
 
@@ -318,7 +332,7 @@ enum {
     SNN_KERNEL_ENCODE = 1,     /* Poisson input spikes and presynaptic traces */
     SNN_KERNEL_NEURON = 2,     /* current, excitatory/inhibitory neurons, postsynaptic traces */
     SNN_KERNEL_STDP = 3,       /* batch-reduced STDP and adaptive thresholds */
-    SNN_KERNEL_PERSISTENT = 4, /* all phases of all steps in one launch */
+    SNN_KERNEL_PERSISTENT = 4, /* all phases of all steps in one launch (of any kernel) */
     SNN_KERNEL_COUNT = 5
 };
 
@@ -331,7 +345,7 @@ SNN_API snn_status snn_profile(snn_net* net, double* ms, int* launches, int n);
 
 /* Tune the automatic choice (SNN_MODE_AUTO) for this network at batch B: runs
  * T steps of each form that takes the run -- the graph of per-step launches,
- * the persistent kernel, and the tensor form with the product and with the
+ * the persistent form, and the tensor form with the product and with the
  * gathered current -- twice each (the first warms up allocation and graph
  * capture), times the second with CUDA events on `cuda_stream`, and restores
  * W and theta before every run and at the end, so tuning leaves them as they

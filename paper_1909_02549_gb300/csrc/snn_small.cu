@@ -3,8 +3,7 @@
 //
 // With few samples a step has little work, and the column kernel's step is a
 // chain of round trips through L2: the grid barrier, the staged counts, lists
-// and masks, the encode's thresholds and traces (784->100 at B = 1: 8.2 us a
-// step, 784->400 at B = 16: 9.1).  Here CTA r of a cluster of CS owns the
+// and masks, the encode's thresholds and traces.  Here CTA r of a cluster of CS owns the
 // columns [r*ncc, (r+1)*ncc) of every sample, and all it needs of the others
 // reaches its shared memory directly: the input-spike words (each CTA draws a
 // share and stores it in every CTA) and the inhibitory counts (a spike adds to
@@ -17,9 +16,10 @@
 //      words.  Arrive at the cluster barrier;
 //   C  the update: a warp per 32 input rows, then wait at the cluster barrier.
 // What bounds it: the instructions of one warp in turn (some twelve cycles each
-// with their stalls, 420 a warp and step at 784->100, B = 1) and the three
-// barriers.  Us a step before and here: 784->100 at B = 1: 7.7 and 2.0,
-// 784->400 at B = 16: 8.6 and 5.3.
+// with their stalls, 420 a warp and step at 784->100, B = 1), the cluster barrier
+// and three block barriers.  Us a step in the column kernel and here, runs of 60
+// steps with their start: 784->100 at B = 1 8.1 and 2.5, 784->400 at B = 16 9.4 and
+// 6.4; each further step 7.7 and 2.0, 8.6 and 5.3.
 //
 // Same sums as the other forms: currents in ascending input, the potentiation
 // and depression sums each in ascending sample; terms left out are +0.
@@ -450,11 +450,10 @@ cudaError_t launch_small(const Consts& c, const Bufs& d, int T, cudaStream_t s, 
     // with 32, the cluster barrier with its stores 865 with 8 CTAs and 1140 to
     // 1240 with 16 (784->100, B = 1: 1024 threads and 16 CTAs 746 us a run of 250
     // steps, 512 and 8 629, 256 and 4 709; 784->400, B = 16: 1024 threads 1441,
-    // 512 1915).  Above ITEMS items a CTA the column kernel is faster (us a step
-    // there and here, 1000 columns of 100 inputs at B = 4 and 8: 9.9 and 10.8,
-    // 6.7 and 11.7; 784->400 at B = 16: 8.6 and 5.3).  Without lateral inhibition the
-    // columns fire in bursts, and each that fired costs a warp a pass over its rows, with
-    // a division each where the mean takes one: fewer items (100 inputs of 120 Hz: 100->
+    // 512 1915).  Above ITEMS items a CTA the column kernel is faster (us a step there
+    // and here, 1000 columns of 100 inputs: B = 4 9.9 and 6.7, B = 8 10.8 and 11.7).
+    // Without lateral inhibition the columns fire in bursts, and each that fired costs a
+    // warp a pass over its rows, with a division each where the mean takes one: fewer items (100 inputs of 120 Hz: 100->
     // 224, B = 32 9.2 and 10.5, 100->6400, B = 1 9.6 and 12.2, 100->280, B = 24 10.3 and
     // 12.8, 100->144, B = 24 10.3 and 10.8; but 100->100, B = 32 9.1 and 8.8, 100->4000, B
     // = 1 9.3 and 7.8, 100->100, B = 17 10.2 and 9.0).  With inhibition, dense inputs cost

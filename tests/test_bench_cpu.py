@@ -184,3 +184,18 @@ def test_reference_arm_prints_the_contract_line():
     assert cb["kind"] == "oracle" and cb["cores"] >= 1 and cb["value"] == d["value"] and cb["sample"]
     assert d["e2e"] == {"value": d["value"], "unit": d["unit"], "h2d_bytes_per_step": 0,
                         "d2h_bytes_per_step": 0}
+
+
+def test_the_drive_kernel_is_not_charged_for_the_spike_counts():
+    import bench
+    p = {"n_in": 1024, "n_hid": 4096, "n_out": 10}
+    assert round(bench.rec_drive_bytes_per_launch(p, 4096) / 1e6, 1) == 411.5
+    assert bench.rec_bytes_per_launch(p, 4096) - bench.rec_drive_bytes_per_launch(p, 4096) == 8 * 4096 * 4096
+
+
+def test_a_profile_names_the_kernel_that_ran():
+    import bench
+    assert bench.kernel_name("persistent", 256, True) == "k_persistent"
+    assert "k_infer" in bench.kernel_name("persistent", 256, False)
+    assert "k_small" in bench.kernel_name("persistent", 16, True)
+    assert bench.kernel_name("neuron", 16, True) == "k_neuron"
